@@ -118,9 +118,13 @@ typedef struct {
                           when max_iter % check_every == 0), else a host-driven
                           loop; both give identical results                  */
     int variant;       /* kernel variant of the fused ADMM algorithms:
-                          0 = automatic: warp strips where the layout allows
-                          them (binary ADMM: two iterations per launch, as 4),
-                          else TMA-staged tiles (Potts, and binary grids
+                          0 = automatic: Potts with at most 16 labels, float32
+                          cost planes and 16-byte aligned rows and planes (odd
+                          widths: rpADMMII, rpADMMI, pADMMI): labels side by
+                          side, two iterations per launch, same results as the
+                          variant that would follow; else warp strips where the
+                          layout allows them (binary ADMM: two iterations per
+                          launch, as 4), else TMA-staged tiles (Potts, and binary grids
                           of at most 2^21 pixels) where rows and planes are
                           16-byte aligned, else shared-memory tiles;
                           1 = shared-memory tiles;
@@ -365,7 +369,7 @@ cmf_status cmf_solve_potts(const float *d_C, int L, const float *d_alpha, float 
 /* ------------------------------------------------------------------------ */
 /* Autotuning (no counterpart in the paper: a launch-configuration search).  */
 /* Solves the problem from a cold start once per candidate configuration --  */
-/* the kernel variant (1, 2, 4 (binary), 8, 16, 32) of the fused ADMM       */
+/* the kernel variant (0 (Potts), 1, 2, 4 (binary), 8, 16, 32) of the fused ADMM */
 /* algorithms, or the sRBGS sweep count (1, 2, 3) of fused rPDRQ, and with   */
 /* p->tune_step = 1 the ADMM step size c (c, 2c, 4c, 8c) -- with everything  */
 /* else taken from *p, and writes the candidate with the shortest time to   */

@@ -465,7 +465,10 @@ struct PottsCall {
     int storage;
     bool tma;                    // fused ADMM through TMA-staged tiles
     bool strip;                  // fused ADMM by warp strips
+    bool rows;                   // fused ADMM, labels side by side, up to two iterations a launch
     PottsTmaMaps maps[2];        // tensor maps of the user / workspace state sets
+    PottsRowsMaps rmaps[2];
+    int rfused;                  // potts_rows_fused
     int* err;                    // sticky device error word
 };
 
@@ -499,8 +502,20 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     call.err = &((SolveCtl*)(call.wsbase + call.w.ctl))->err;
     call.tma = false;
     call.strip = false;
-    // automatic choice: warp strips where the layout allows them (fastest on
-    // every measured Potts case), else TMA tiles, else shared-memory tiles
+    call.rows = false;
+    // automatic choice: labels side by side (two iterations a launch; against
+    // the strips 150 -> 64 us per iteration at 2048^2, L = 4 and 2293 -> 968 us
+    // at 4096^2, L = 16, faster at every size measured from 128^2 and L = 2 on,
+    // with the same results), else warp strips where the layout allows them,
+    // else TMA tiles, else shared-memory tiles
+    if (!call.cfg.plain && !call.cfg.dr && p->variant == 0 &&
+        potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws) &&
+        potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
+        potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess) {
+        call.rows = true;
+        call.rfused = potts_rows_fused(call.P, p->storage, call.cfg.aniso);
+        return CMF_OK;
+    }
     if (!call.cfg.plain && (p->variant == 2 || p->variant == 4 || p->variant == 0)) {
         const bool ok = potts_strip_eligible(call.P.g, p->storage, C, alpha, call.user, call.ws);
         if (!ok && p->variant != 0)
@@ -527,9 +542,38 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
 }
 
 // As binary_run: n iterations from buffer set `cur` (0 or 1); cert: certify
-// the result with that tail; dry: only follow the buffer sets.
+// the result with that tail; dry: only follow the buffer sets.  home: with
+// two iterations a launch, make the number of launches even where that costs
+// one launch more (less than copying a state set back).
 cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int k0 = 0,
-                      const EvalTail* cert = nullptr, bool dry = false) {
+                      const EvalTail* cert = nullptr, bool dry = false, bool home = false) {
+    if (c.rows && n > 0) {
+        // single launches for the scheduled iterations and an odd remainder
+        const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
+        int singles = sched < n ? sched : n;
+        singles += (n - singles) % 2;
+        if (home && singles + 2 <= n && (singles + (n - singles) / 2) % 2) singles += 2;
+        float cu_in = 0.0f;  // the first launch reads u itself, later ones the w form
+        for (int i = 0; i < n;) {
+            const int it = i < singles ? 1 : 2;
+            if (!dry) {
+                const StepConfig cfg = step_at(c.cfg, c.prm, c.P.L, true, k0 + i);
+                cudaError_t e =
+                    potts_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso, cfg.ac,
+                                    cu_in, it, c.rmaps[cur], c.rfused, c.err, st);
+                if (e != cudaSuccess) return e;
+            }
+            cu_in = c.cfg.ac.cu;
+            cur ^= 1;
+            i += it;
+        }
+        if (!dry) {
+            cudaError_t e = potts_strip_finalize(c.storage, c.P, cur == 0 ? c.user : c.ws,
+                                                 c.cfg.ac.cu, st);
+            if (e != cudaSuccess) return e;
+        }
+        n = 0;
+    }
     if (dry) {
         if (n > 0) cur = c.cfg.plain ? 0 : (n % 2 ? cur ^ 1 : cur);
         return cudaSuccess;
@@ -1143,7 +1187,7 @@ cmf_status cmf_iterate_potts(const float* d_C, int L, const float* d_alpha, floa
     cudaStream_t st = (cudaStream_t)stream;
     CMF_CUDA_TRY(cudaMemsetAsync(c.err, 0, sizeof(int), st));
     int cur = 0;
-    CMF_CUDA_TRY(potts_run(c, n_iter, cur, st));
+    CMF_CUDA_TRY(potts_run(c, n_iter, cur, st, 0, nullptr, false, true));
     if (cur != 0) CMF_CUDA_TRY(copy_potts(c.user, c.ws, c.P.g, L, c.storage, st));
     return CMF_OK;
 }
@@ -1274,7 +1318,7 @@ std::vector<cmf_params> tune_candidates(const cmf_params& p, bool binary) {
     std::vector<int> variants = {p.variant};
     std::vector<int> sweeps = {p.sweeps};
     if (fused && !dr) variants = binary ? std::vector<int>{1, 2, 4, 8, 16, 32}
-                                        : std::vector<int>{1, 2, 8, 16, 32};
+                                        : std::vector<int>{0, 1, 2, 8, 16, 32};
     if (fused && dr) sweeps = {1, 2, 3};
     for (int v : variants)
         for (int s : sweeps) {

@@ -396,6 +396,27 @@ cudaError_t potts_dr_strip_step(int storage, const PottsProblem& P, const PottsS
 cudaError_t potts_strip_finalize(int storage, const PottsProblem& P, const PottsStateV& s,
                                  float cu, cudaStream_t st);
 
+// --- Potts ADMM, labels side by side (cmf_potts_rows.cuh) ---
+// Tensor maps of one state set and of the problem's planes.
+struct PottsRowsMaps {
+    CUtensorMap qx, qy, p, u, ps, C, al;
+};
+// Eligible: at most 16 labels, float32 cost planes, 16-byte aligned rows and
+// planes; odd widths under the relaxed ADMM algorithms.
+bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
+                         const PottsStateV& a, const PottsStateV& b);
+// For odd widths, whether the tile kernel that would otherwise run (its
+// 16-row instantiations do, its 8-row ones do not) rounds products into sums.
+int potts_rows_fused(const PottsProblem& P, int storage, bool aniso);
+cudaError_t potts_rows_maps(const PottsProblem& P, int storage, const PottsStateV& s,
+                            PottsRowsMaps& m);
+// `iters` (1 or 2) iterations from the state of src_maps into b, with the
+// multiplier form of potts_strip_step; a bounded wait that runs out sets *err.
+cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsStateV& b, bool aniso,
+                            const AdmmCoef& K, float cu_in, int iters,
+                            const PottsRowsMaps& src_maps, int fused, int* err,
+                            cudaStream_t st);
+
 // --- TMA-staged Potts ADMM (cmf_potts_tma.cu) ---
 struct PottsTmaMaps {
     CUtensorMap qx, qy, p, u, ps;

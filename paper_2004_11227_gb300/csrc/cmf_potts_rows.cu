@@ -1,0 +1,97 @@
+// Host side of the Potts ADMM kernel that runs the labels side by side
+// (cmf_potts_rows.cuh): which layouts it takes, its tensor maps, and the
+// dispatch to the storage type's translation unit.
+#include <climits>
+
+#include "cmf_potts_rows.cuh"
+
+namespace cmf {
+
+cudaError_t potts_rows_step_f32(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                const AdmmCoef& K, float cu_in, int iters,
+                                const PottsRowsMaps& M, int* err, cudaStream_t st);
+cudaError_t potts_rows_tile_step_f32(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                     const AdmmCoef& K, float cu_in, int iters,
+                                     const PottsRowsMaps& M, int fused, int* err,
+                                     cudaStream_t st);
+cudaError_t potts_rows_step_f16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                const AdmmCoef& K, float cu_in, int iters,
+                                const PottsRowsMaps& M, int* err, cudaStream_t st);
+cudaError_t potts_rows_tile_step_f16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                     const AdmmCoef& K, float cu_in, int iters,
+                                     const PottsRowsMaps& M, int fused, int* err,
+                                     cudaStream_t st);
+cudaError_t potts_rows_step_bf16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                 const AdmmCoef& K, float cu_in, int iters,
+                                 const PottsRowsMaps& M, int* err, cudaStream_t st);
+cudaError_t potts_rows_tile_step_bf16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                                      const AdmmCoef& K, float cu_in, int iters,
+                                      const PottsRowsMaps& M, int fused, int* err,
+                                      cudaStream_t st);
+
+bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
+                         const PottsStateV& a, const PottsStateV& b) {
+    const Grid& G = P.g;
+    if (G.W % 2 && (K.ty || K.cp)) return false;
+    if (P.L > rows::kMaxLabels || cost_src(P) != kCostF32) return false;
+    // the last pair of an odd width writes its first element alone, every
+    // other one a pair at an even offset
+    if (G.plane > (size_t)INT_MAX || G.plane * (size_t)P.L > (size_t)UINT_MAX) return false;
+    const size_t es = dtype_size(storage);
+    if ((G.pitch * es) % 16 || (G.pitch * 4) % 16) return false;
+    auto al = [](const void* p) { return ((uintptr_t)p % 16) == 0; };
+    if (!al(P.C) || (P.alpha.plane && !al(P.alpha.plane))) return false;
+    for (const PottsStateV* s : {&a, &b})
+        if (!al(s->u) || !al(s->qx) || !al(s->qy) || !al(s->p) || !al(s->ps)) return false;
+    return true;
+}
+
+int potts_rows_fused(const PottsProblem& P, int storage, bool aniso) {
+    return P.g.W % 2 ? potts_tma_auto_ty(storage, aniso, P.L) == 16 : 0;
+}
+
+cudaError_t potts_rows_maps(const PottsProblem& P, int storage, const PottsStateV& s,
+                            PottsRowsMaps& m) {
+    const Grid& G = P.g;
+    const int es = (int)dtype_size(storage);
+    const int cs = es == 4 ? rows::Seg<4>::cols : rows::Seg<2>::cols, c4 = rows::Seg<4>::cols;
+    const struct {
+        CUtensorMap* map;
+        const void* base;
+        int es, planes, box;
+    } f[7] = {{&m.qx, s.qx, es, P.L, cs}, {&m.qy, s.qy, es, P.L, cs}, {&m.p, s.p, es, P.L, cs},
+              {&m.u, s.u, 4, P.L, c4},    {&m.ps, s.ps, 4, 1, c4},    {&m.C, P.C, 4, P.L, c4},
+              {&m.al, P.alpha.plane, 4, 1, c4}};
+    for (const auto& q : f) {
+        if (!q.base) {  // constant alpha: its map is never read
+            *q.map = m.ps;
+            continue;
+        }
+        const cudaError_t e = encode_tma_3d(q.map, q.base, q.es, G.W, G.H, q.planes, G.pitch,
+                                            q.box, 1, q.planes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsStateV& b, bool aniso,
+                            const AdmmCoef& K, float cu_in, int iters, const PottsRowsMaps& M,
+                            int fused, int* err, cudaStream_t st) {
+    if (P.g.W % 2) {
+        switch (storage) {
+            case CMF_F32:
+                return potts_rows_tile_step_f32(P, b, aniso, K, cu_in, iters, M, fused, err, st);
+            case CMF_F16:
+                return potts_rows_tile_step_f16(P, b, aniso, K, cu_in, iters, M, fused, err, st);
+            default:
+                return potts_rows_tile_step_bf16(P, b, aniso, K, cu_in, iters, M, fused, err, st);
+        }
+    }
+    switch (storage) {
+        case CMF_F32: return potts_rows_step_f32(P, b, aniso, K, cu_in, iters, M, err, st);
+        case CMF_F16: return potts_rows_step_f16(P, b, aniso, K, cu_in, iters, M, err, st);
+        default: return potts_rows_step_bf16(P, b, aniso, K, cu_in, iters, M, err, st);
+    }
+}
+
+}  // namespace cmf

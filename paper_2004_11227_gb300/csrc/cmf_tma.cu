@@ -20,7 +20,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 cudaError_t encode_tma_3d(CUtensorMap* map, const void* base, int elem_bytes, int cols, int rows,
-                          int planes, int pitch, int box_x, int box_y) {
+                          int planes, int pitch, int box_x, int box_y, int box_z) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return cudaErrorInvalidValue;
     // plain bit copies: unsigned types of the element width (out-of-range
@@ -30,7 +30,8 @@ cudaError_t encode_tma_3d(CUtensorMap* map, const void* base, int elem_bytes, in
     const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)pitch * elem_bytes,
                                    (cuuint64_t)pitch * elem_bytes * (cuuint64_t)rows};
-    const cuuint32_t box[3] = {(cuuint32_t)box_x, (cuuint32_t)box_y, 1u};
+    const cuuint32_t box[3] = {(cuuint32_t)box_x, (cuuint32_t)box_y,
+                               (cuuint32_t)box_z};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     CUresult r = fn(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

@@ -97,9 +97,9 @@ constexpr long long kWaitLimitCycles = 2000000000ll;
 
 // Encode a row-major [planes][rows][cols] tensor of `elem_bytes` elements with
 // a row stride of `pitch` elements and a plane stride of rows * pitch; box
-// {box_x, box_y, 1}; out-of-range elements read as zero.  Returns
+// {box_x, box_y, box_z}; out-of-range elements read as zero.  Returns
 // cudaErrorInvalidValue when the driver rejects the description.
 cudaError_t encode_tma_3d(CUtensorMap* map, const void* base, int elem_bytes, int cols, int rows,
-                          int planes, int pitch, int box_x, int box_y);
+                          int planes, int pitch, int box_x, int box_y, int box_z = 1);
 
 }  // namespace cmf
