@@ -118,24 +118,26 @@ typedef struct {
                           when max_iter % check_every == 0), else a host-driven
                           loop; both give identical results                  */
     int variant;       /* kernel variant of the fused ADMM algorithms:
-                          0 = automatic: Potts with at most 16 labels, float32
-                          cost planes and 16-byte aligned rows and planes (odd
-                          widths: rpADMMII, rpADMMI, pADMMI): labels side by
-                          side, two iterations per launch, same results as the
-                          variant that would follow; else warp strips where the
-                          layout allows them (binary ADMM: two iterations per
-                          launch, as 4), else TMA-staged tiles (Potts, and binary grids
+                          0 = automatic: where rows and planes are 16-byte
+                          aligned, binary: chains of warps, up to four
+                          iterations per launch; Potts with at most 16 labels
+                          and float32 cost planes (odd widths: rpADMMII,
+                          rpADMMI, pADMMI): labels side by side, two iterations
+                          per launch; both with the results of the variant that
+                          would follow: warp strips where the layout allows
+                          them (binary ADMM: two iterations per launch), else
+                          TMA-staged tiles (Potts, and binary grids
                           of at most 2^21 pixels) where rows and planes are
                           16-byte aligned, else shared-memory tiles;
                           1 = shared-memory tiles;
                           2 = warp strips (even W and pitch, planes aligned to
                           two elements; for Potts the multipliers are kept as
                           u - cu p_s between the iterations of one call);
-                          4 = binary ADMM: warp strips making two iterations
-                          per launch (the intermediate state stays on chip;
-                          an even number of such launches per call, single
-                          ones for the rest and for scheduled rho_k; same
-                          results as 2); Potts and rPDRQ: as 2;
+                          4 = binary ADMM, even widths: as 0 (chains of warps,
+                          else warp strips making two iterations per launch,
+                          the intermediate state on chip; single ones for an
+                          odd rest and for scheduled rho_k; float32 results as
+                          2); Potts and rPDRQ: as 2;
                           8 / 16 / 32 = TMA tiles of that many rows         */
     double c;          /* ADMM step size                                       */
     double a;          /* q preconditioner N = a c I (a >= 8, Thm 1)           */

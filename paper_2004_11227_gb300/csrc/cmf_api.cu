@@ -211,6 +211,9 @@ struct BinaryCall {
     bool tma;               // fused ADMM through the persistent TMA kernel
     bool strip;             // fused ADMM by warp strips
     bool pairs;             // warp strips, two ADMM iterations per launch
+    bool chain;             // chains of warps, up to four ADMM iterations per launch
+    BinChainMaps cmaps[3];  // tensor maps of the buffer sets
+    int cert_blocks;        // partial triples the workspace holds
     BinTmaMaps maps[2];     // tensor maps of the user / workspace state sets
     int* err;               // sticky device error word
 };
@@ -246,9 +249,23 @@ cmf_status binary_prepare(const float* Cs, const float* Ct, const float* alpha, 
     call.tma = false;
     call.strip = false;
     call.pairs = false;
-    // automatic choice: warp strips where the layout allows them, two ADMM
-    // iterations per launch (1.5x faster per iteration than one at 1024^2,
-    // 1.9x at 4096^2, which beats the persistent TMA kernel: measured);
+    call.chain = false;
+    // automatic choice: chains of warps (against pairs of iterations by warp
+    // strips 8.25 -> 5.73 us per iteration at 1024^2, 87 -> 52 us at 4096^2;
+    // odd widths, against tiles, 16 -> 7.2 us at 901 x 1407; the same results)
+    if (!call.cfg.plain && !call.cfg.dr &&
+        (p->variant == 0 || (p->variant == 4 && W % 2 == 0)) &&
+        binary_chain_eligible(call.P, p->storage, call.user, call.ws, call.ws2) &&
+        binary_chain_maps(call.P, p->storage, call.user, call.cmaps[0]) == cudaSuccess &&
+        binary_chain_maps(call.P, p->storage, call.ws, call.cmaps[1]) == cudaSuccess &&
+        binary_chain_maps(call.P, p->storage, call.ws2, call.cmaps[2]) == cudaSuccess) {
+        call.chain = true;
+        const int nb = eval_blocks(H, W), nc = binary_cert_max_blocks();
+        call.cert_blocks = nb > nc ? nb : nc;
+        return CMF_OK;
+    }
+    // else warp strips where the layout allows them, two ADMM iterations per
+    // launch (1.5x faster per iteration than one at 1024^2, 1.9x at 4096^2);
     // rPDRQ: the pipelined red-black sweeps
     if (!call.cfg.plain && (p->variant == 2 || p->variant == 4 || p->variant == 0)) {
         const bool ok =
@@ -300,6 +317,37 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
     // -> start, x and y the other two sets; a lone launch goes to the
     // caller's set, or from it to the workspace.
     int i = 0;
+    if (c.chain) {
+        // one iteration per launch while the rho schedule lasts, then launches
+        // of up to four iterations, at least two of them; the last one carries
+        // the certificates
+        const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
+        const int first = sched < n ? sched : n;
+        const bool may_cert = cert && binary_chain_certifies(c.P.g, c.cert_blocks);
+        const int rest = n - first, most = binary_chain_max_iters();
+        int nl = rest < 2 ? rest : (rest + most - 1) / most;  // launches of the rest
+        if (nl == 1 && rest > 1) nl = 2;
+        int start = cur;
+        for (int j = 0; j < first + nl; ++j) {
+            const int m = j - first;  // m >= 0: a launch of the rest
+            if (m <= 0) start = cur;
+            const int x = start == 0 ? 1 : 0, y = start == 2 ? 1 : 2;
+            const int T = m < 0 ? 1 : rest / nl + (m < rest % nl ? 1 : 0);
+            const int dst = m < 0 || nl == 1 ? (cur == 0 ? 1 : 0)
+                                             : (m == nl - 1 ? start : (m % 2 == 0 ? x : y));
+            certified = may_cert && j == first + nl - 1;
+            if (!dry) {
+                const StepConfig cfg = m < 0 ? step_at(c.cfg, c.prm, 2, false, k0 + j) : c.cfg;
+                cudaError_t e = binary_chain_step(c.storage, c.P, bset(c, dst), cfg.aniso, cfg.ac,
+                                                  T, i, c.cmaps[cur], partials, c.cert_blocks,
+                                                  certified ? cert : nullptr, c.err, st);
+                if (e != cudaSuccess) return e;
+            }
+            if (m >= 0) i += T;
+            cur = dst;
+        }
+        i = n;
+    }
     if (c.pairs) {
         const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
         const int first = sched < n ? sched : n;

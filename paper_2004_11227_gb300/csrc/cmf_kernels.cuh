@@ -370,6 +370,28 @@ cudaError_t binary_eval_strip(int storage, const BinProblem& P, const BinStateV&
                               bool dr, float tau, double* partials, cudaStream_t st,
                               const EvalTail& T);
 
+// --- binary ADMM by chains of warps (cmf_binary_chain.cuh) ---
+// Tensor maps of one state set and of the problem's planes.
+struct BinChainMaps {
+    CUtensorMap qx, qy, ps, pt, u, Cs, Ct, al;
+};
+int binary_chain_max_iters();  // per launch
+// Eligible: 16-byte aligned rows and planes; any width.
+bool binary_chain_eligible(const BinProblem& P, int storage, const BinStateV& a,
+                           const BinStateV& b, const BinStateV& c);
+// Whether a launch can certify its result with at most max_blocks partials.
+bool binary_chain_certifies(const Grid& G, int max_blocks);
+cudaError_t binary_chain_maps(const BinProblem& P, int storage, const BinStateV& s,
+                              BinChainMaps& m);
+// T iterations (1 .. binary_chain_max_iters) from the state of src_maps into
+// b; iter0: the first one's index among the call's unscheduled iterations;
+// cert: as binary_strip2_step, with at most max_blocks partial triples; a
+// bounded wait that runs out sets *err.
+cudaError_t binary_chain_step(
+    int storage, const BinProblem& P, const BinStateV& b, bool aniso, const AdmmCoef& K, int T,
+    int iter0, const BinChainMaps& src_maps, double* partials, int max_blocks, const EvalTail* cert, int* err,
+    cudaStream_t st);
+
 // --- warp-strip Potts ADMM (cmf_potts_strip.cu) ---
 // Eligible: even W and pitch, H * pitch within int, pair-aligned planes.
 // odd_width_ok: the ADMM items of a batch also take odd widths (their last
