@@ -324,9 +324,10 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
         const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
         const int first = sched < n ? sched : n;
         const bool may_cert = cert && binary_chain_certifies(c.P.g, c.cert_blocks);
-        const int rest = n - first, most = binary_chain_max_iters();
+        const int rest = n - first, most = binary_chain_max_iters(false);
         int nl = rest < 2 ? rest : (rest + most - 1) / most;  // launches of the rest
         if (nl == 1 && rest > 1) nl = 2;
+        if (may_cert && rest > 0 && rest / nl > binary_chain_max_iters(true)) ++nl;
         int start = cur;
         for (int j = 0; j < first + nl; ++j) {
             const int m = j - first;  // m >= 0: a launch of the rest
@@ -514,6 +515,7 @@ struct PottsCall {
     bool tma;                    // fused ADMM through TMA-staged tiles
     bool strip;                  // fused ADMM by warp strips
     bool rows;                   // fused ADMM, labels side by side, up to two iterations a launch
+    bool cert;                   // certificates with the labels side by side
     PottsTmaMaps maps[2];        // tensor maps of the user / workspace state sets
     PottsRowsMaps rmaps[2];
     int rfused;                  // potts_rows_fused
@@ -556,10 +558,11 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     // at 4096^2, L = 16, faster at every size measured from 128^2 and L = 2 on,
     // with the same results), else warp strips where the layout allows them,
     // else TMA tiles, else shared-memory tiles
-    if (!call.cfg.plain && !call.cfg.dr && p->variant == 0 &&
-        potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws) &&
-        potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
-        potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess) {
+    call.cert = potts_rows_layout(call.P, p->storage, call.user, call.ws) &&
+                potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
+                potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess;
+    if (!call.cfg.plain && !call.cfg.dr && p->variant == 0 && call.cert &&
+        potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws)) {
         call.rows = true;
         call.rfused = potts_rows_fused(call.P, p->storage, call.cfg.aniso);
         return CMF_OK;
@@ -587,6 +590,19 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     if (!call.tma && !call.cfg.dr && !call.cfg.plain && p->variant >= 8)
         return CMF_EINVAL;  // TMA tiles requested but the layout does not allow them
     return CMF_OK;
+}
+
+// The certificate launch for buffer set `set` (0 or 1): labels side by side
+// where the layout allows it (a call, host part included: 2048^2, L = 16
+// 547 -> 423 us, L = 4 197 -> 153 us; 721 x 1283, L = 8 199 -> 97 us; not
+// slower anywhere from 128^2 on), else the strip or tile kernel.
+cudaError_t potts_certify(const PottsCall& c, int set, cudaStream_t st, const EvalTail& T) {
+    double* partials = (double*)(c.wsbase + c.w.partials);
+    if (c.cert)
+        return potts_cert(c.storage, c.P, c.rmaps[set], c.cfg.aniso, c.cfg.dr, c.cfg.dc.tau,
+                          partials, T, c.err, st);
+    return potts_eval(c.storage, c.P, set == 0 ? c.user : c.ws, c.cfg.aniso, c.cfg.dr,
+                      c.cfg.dc.tau, partials, st, T);
 }
 
 // As binary_run: n iterations from buffer set `cur` (0 or 1); cert: certify
@@ -671,18 +687,13 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
             cur ^= 1;
         }
     }
-    if (cert)
-        return potts_eval(c.storage, c.P, cur == 0 ? c.user : c.ws, c.cfg.aniso, c.cfg.dr,
-                          c.cfg.dc.tau, (double*)(c.wsbase + c.w.partials), st, *cert);
-    return cudaSuccess;
+    return cert ? potts_certify(c, cur, st, *cert) : cudaSuccess;
 }
 
-cmf_status potts_eval_state(const PottsCall& c, const PottsStateV& s, double* h_out,
-                            cudaStream_t st) {
+cmf_status potts_eval_state(const PottsCall& c, double* h_out, cudaStream_t st) {
     const EvalTail T = reduce_tail(c.wsbase, c.w);
     CMF_CUDA_TRY(cudaMemsetAsync(&T.ctl->arrive, 0, sizeof(unsigned), st));
-    CMF_CUDA_TRY(potts_eval(c.storage, c.P, s, c.cfg.aniso, c.cfg.dr, c.cfg.dc.tau,
-                            (double*)(c.wsbase + c.w.partials), st, T));
+    CMF_CUDA_TRY(potts_certify(c, 0, st, T));
     return finish_eval(c.wsbase, c.w, h_out, st);
 }
 
@@ -1250,7 +1261,7 @@ cmf_status cmf_eval_potts(const float* d_C, int L, const float* d_alpha, float a
                                  (void*)d_qx, (void*)d_qy, (void*)d_p, (void*)d_ps, d_ws,
                                  ws_bytes, c);
     if (s != CMF_OK) return s;
-    return potts_eval_state(c, c.user, h_out, (cudaStream_t)stream);
+    return potts_eval_state(c, h_out, (cudaStream_t)stream);
 }
 
 // The first phase of a two-phase solve also ends when its certified gap,

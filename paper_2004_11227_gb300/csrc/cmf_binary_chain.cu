@@ -18,7 +18,7 @@ cudaError_t binary_chain_step_bf16(
     const AdmmCoef& K, int T, int iter0, const BinChainMaps& M, double* partials, int max_blocks,
     const EvalTail* cert, int* err, cudaStream_t st);
 
-int binary_chain_max_iters() { return chain::kMaxIters; }
+int binary_chain_max_iters(bool cert) { return cert ? chain::kMaxCert : chain::kMaxIters; }
 
 bool binary_chain_eligible(const BinProblem& P, int storage, const BinStateV& a,
                            const BinStateV& b, const BinStateV& c) {
@@ -34,8 +34,8 @@ bool binary_chain_eligible(const BinProblem& P, int storage, const BinStateV& a,
 }
 
 bool binary_chain_certifies(const Grid& G, int max_blocks) {
-    const int out = chain::kCols - chain::left_cols(chain::kMaxIters) -
-                    chain::right_cols(chain::kMaxIters, true);
+    const int out = chain::kCols - chain::left_cols(chain::kMaxCert) -
+                    chain::right_cols(chain::kMaxCert, true);
     return (G.W + out - 1) / out <= max_blocks;
 }
 

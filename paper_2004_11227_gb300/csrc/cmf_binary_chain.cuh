@@ -10,8 +10,9 @@
 // and alpha, come by TMA (elements outside the grid read as zero); the rows
 // between two warps pass through shared memory, two slots each, in the storage
 // type as a store and a load would round them; the last warp writes the
-// result.  With CERT a further warp sums the certificates of the rows the last
-// one makes.  A producer warp keeps kIn rows in flight and waits for each row
+// result.  With CERT two further warps sum the certificates of the rows the
+// last one makes (one the energy, one the dual value and the residual: either
+// is about an iteration's work).  A producer warp keeps kIn rows in flight and waits for each row
 // before the step that reads it, so the one block barrier per step is all the
 // other warps wait on:
 //   - a slot between two warps is written in one step, read in the next and
@@ -52,7 +53,7 @@ namespace chain {
 
 using strip::Pair;
 
-constexpr int kMaxIters = 4;  // iterations per launch
+constexpr int kMaxIters = 4, kMaxCert = 3;  // iterations per launch, and with certificates
 constexpr int kAux = 16;      // C_s / C_t / alpha rows in shared memory
 constexpr int kIn = 4;        // input rows in flight
 constexpr int kCols = 128;    // columns of a strip
@@ -160,7 +161,7 @@ __device__ __forceinline__ void project(float& x, float& y, float al, bool swap)
 // their pairs does at even ones too (iter0: the call's index of warp 0's
 // iteration).
 template <typename S, bool ANISO, bool SIMPLE, bool EVEN, bool CERT>
-__global__ void __launch_bounds__(32 * (chain::kMaxIters + 1 + (CERT ? 1 : 0)), CERT ? 3 : 4)
+__global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMaxIters + 1), CERT ? 3 : 4)
     k_binary_chain(const __grid_constant__ BinChainMaps M, BinProblem Pr, BinState<S> s1,
                    AdmmCoef K, int T, int iter0, int R, int nstrips, double* partials,
                    EvalTail tail, int* err) {
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(32 * (chain::kMaxIters + 1 + (CERT ? 1 : 0)), 
     __syncthreads();
 
     DF accE = {0.f, 0.f}, accD = {0.f, 0.f}, accR = {0.f, 0.f};
-    if (wib == T + (CERT ? 1 : 0)) {
+    if (wib == T + (CERT ? 2 : 0)) {
         // ---- producer ------------------------------------------------------
         const uint32_t tx = 4u * Seg<ES>::row + (has_al ? 4u : 3u) * Seg<4>::row;
         const int xs = cfirst - offs;
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(32 * (chain::kMaxIters + 1 + (CERT ? 1 : 0)), 
                 mbar_wait_bounded(bar + i, 1, kWaitLimitCycles);
             }
     } else {
-        const int t = wib;
+        const int t = min(wib, T);  // place in the chain
         // 0/1 weights of the x differences (0 left of the grid, at the last
         // column and right of it); only a strip's edges have zeros
         float mx[4];
@@ -422,58 +423,89 @@ __global__ void __launch_bounds__(32 * (chain::kMaxIters + 1 + (CERT ? 1 : 0)), 
             }
         } else {
             // ---- certificates of the rows the last iteration makes ---------
-            // (primal energy E at clip(u, 0, 1), dual value D of the
-            // re-projected flows, squared conservation residual)
-            F4 py_up = zero, qn_up = zero;  // q_y of the row above, projected and as it is
+            const int sa = 3 * T - 2;
+            if (wib == T) {
+                // primal energy E at clip(u, 0, 1)
+                const unsigned char* const ru = rd + mu;
+                F4 un = zero;
 #pragma unroll 1
-            for (int s = -2; s <= se; ++s) {
-                __syncthreads();
-                if (s >= 3 * T - 2) {
-                    x[0] = x[1];
-                    load((s & 1) ^ 1, x[1]);
-                    const unsigned char* a = ax + arow * Y::aux;
-                    const F4 cs = QF::f4(QF::ld(a)), ct = QF::f4(QF::ld(a + Y::f4)),
-                             al = QF::f4(QF::ld(a + 2 * Y::f4));
-                    const float wy = row_w(r);
-                    const F4 qx = QS::f4(x[0].qx), qy = QS::f4(x[0].qy);
-                    F4 px = qx, py = qy, ub = QF::f4(x[0].u), ud = QF::f4(x[1].u);
+                for (int s = -2; s <= se; ++s) {
+                    __syncthreads();
+                    if (s >= sa) {
+                        F4 ub = un;
+                        un = QF::f4(QF::ld(ru + ((s & 1) ^ 1) * Y::mid));
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        project<ANISO>(px.v[i], py.v[i], al.v[i], EVEN && (i & 1));
-                        ub.v[i] = __saturatef(ub.v[i]);
-                        ud.v[i] = __saturatef(ud.v[i]);
-                    }
-                    const F4 d = div_of(qx, qy, wy, qn_up), dp = div_of(px, py, wy, py_up);
-                    const float ubr = right_of(ub.v[0]);
-                    if (own && r >= r0 && r < r1) {
-                        const F4 ps = QS::f4(x[0].ps), pt = QS::f4(x[0].pt);
+                        for (int i = 0; i < 4; ++i) un.v[i] = __saturatef(un.v[i]);
+                        const float ubr = right_of(ub.v[0]);
+                        if (own && r >= r0 && r < r1) {
+                            const unsigned char* a = ax + arow * Y::aux;
+                            const F4 cs = QF::f4(QF::ld(a)), ct = QF::f4(QF::ld(a + Y::f4)),
+                                     al = QF::f4(QF::ld(a + 2 * Y::f4));
+                            const float wy = row_w(r);
 #pragma unroll
-                        for (int h = 0; h < 4; h += 2) {  // a pair's terms together
-                            float e = 0.f, r2 = 0.f, m = 0.f, tv = 0.f;
+                            for (int h = 0; h < 4; h += 2) {  // a pair's terms together
+                                float e = 0.f, tv = 0.f;
 #pragma unroll
-                            for (int i = h; i < h + 2; ++i) {
-                                if (c + i >= G.W) continue;
-                                const float gx =
-                                    mx[i] * ((i < 3 ? ub.v[i < 3 ? i + 1 : 3] : ubr) - ub.v[i]);
-                                const float gy = wy * (ud.v[i] - ub.v[i]);
-                                tv += al.v[i] *
-                                      (ANISO ? fabsf(gx) + fabsf(gy) : sqrtf(gx * gx + gy * gy));
-                                e += (1.f - ub.v[i]) * cs.v[i] + ub.v[i] * ct.v[i];
-                                const float res = d.v[i] - ps.v[i] + pt.v[i];
-                                r2 += res * res;
-                                m += fminf(cs.v[i], ct.v[i] + dp.v[i]);
+                                for (int i = h; i < h + 2; ++i) {
+                                    if (c + i >= G.W) continue;
+                                    const float gx =
+                                        mx[i] *
+                                        ((i < 3 ? ub.v[i < 3 ? i + 1 : 3] : ubr) - ub.v[i]);
+                                    const float gy = wy * (un.v[i] - ub.v[i]);
+                                    tv += al.v[i] * (ANISO ? fabsf(gx) + fabsf(gy)
+                                                           : sqrtf(gx * gx + gy * gy));
+                                    e += (1.f - ub.v[i]) * cs.v[i] + ub.v[i] * ct.v[i];
+                                }
+                                df_add(accE, tv);
+                                df_add(accE, e);
                             }
-                            df_add(accE, tv);
-                            df_add(accE, e);
-                            df_add(accR, r2);
-                            df_add(accD, m);
                         }
                     }
-                    py_up = py;
-                    qn_up = qy;
+                    ++r;
+                    arow = (arow + 1) & (kAux - 1);
                 }
-                ++r;
-                arow = (arow + 1) & (kAux - 1);
+            } else {
+                // dual value D of the re-projected flows, squared residual
+                F4 py_up = zero, qn_up = zero;  // q_y of the row above, projected and as it is
+#pragma unroll 1
+                for (int s = -2; s <= se; ++s) {
+                    __syncthreads();
+                    if (s > sa) {
+                        // row r: the slot the last iteration wrote two steps ago
+                        // is being rewritten, so the row was kept
+                        const unsigned char* a = ax + arow * Y::aux;
+                        const F4 al = QF::f4(QF::ld(a + 2 * Y::f4));
+                        const float wy = row_w(r);
+                        const F4 qx = QS::f4(x[0].qx), qy = QS::f4(x[0].qy);
+                        F4 px = qx, py = qy;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            project<ANISO>(px.v[i], py.v[i], al.v[i], EVEN && (i & 1));
+                        const F4 d = div_of(qx, qy, wy, qn_up), dp = div_of(px, py, wy, py_up);
+                        if (own && r >= r0 && r < r1) {
+                            const F4 ps = QS::f4(x[0].ps), pt = QS::f4(x[0].pt);
+                            const F4 cs = QF::f4(QF::ld(a)), ct = QF::f4(QF::ld(a + Y::f4));
+#pragma unroll
+                            for (int h = 0; h < 4; h += 2) {
+                                float r2 = 0.f, m = 0.f;
+#pragma unroll
+                                for (int i = h; i < h + 2; ++i) {
+                                    if (c + i >= G.W) continue;
+                                    const float res = d.v[i] - ps.v[i] + pt.v[i];
+                                    r2 += res * res;
+                                    m += fminf(cs.v[i], ct.v[i] + dp.v[i]);
+                                }
+                                df_add(accR, r2);
+                                df_add(accD, m);
+                            }
+                        }
+                        py_up = py;
+                        qn_up = qy;
+                    }
+                    if (s >= sa) load((s & 1) ^ 1, x[0]);
+                    ++r;
+                    arow = (arow + 1) & (kAux - 1);
+                }
             }
         }
     }
@@ -498,7 +530,7 @@ static cudaError_t launch_binary_chain(const BinProblem& P, const BinState<S>& b
     if (e != cudaSuccess) return e;
     // blocks resident per device and chain length
     static std::atomic<long long> memo[chain::kMaxIters + 1][kMaxDevices];
-    const int threads = 32 * (T + 1 + (CERT ? 1 : 0));
+    const int threads = 32 * (T + (CERT ? 3 : 1));
     long long resident = 0;
     e = per_device(
         memo[T],

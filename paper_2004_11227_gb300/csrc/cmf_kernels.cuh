@@ -375,7 +375,7 @@ cudaError_t binary_eval_strip(int storage, const BinProblem& P, const BinStateV&
 struct BinChainMaps {
     CUtensorMap qx, qy, ps, pt, u, Cs, Ct, al;
 };
-int binary_chain_max_iters();  // per launch
+int binary_chain_max_iters(bool cert);  // per launch
 // Eligible: 16-byte aligned rows and planes; any width.
 bool binary_chain_eligible(const BinProblem& P, int storage, const BinStateV& a,
                            const BinStateV& b, const BinStateV& c);
@@ -423,8 +423,11 @@ cudaError_t potts_strip_finalize(int storage, const PottsProblem& P, const Potts
 struct PottsRowsMaps {
     CUtensorMap qx, qy, p, u, ps, C, al;
 };
-// Eligible: at most 16 labels, float32 cost planes, 16-byte aligned rows and
-// planes; odd widths under the relaxed ADMM algorithms.
+// The layouts these kernels take: at most 16 labels, float32 cost planes,
+// 16-byte aligned rows and planes; any width.
+bool potts_rows_layout(const PottsProblem& P, int storage, const PottsStateV& a,
+                       const PottsStateV& b);
+// The iterations they take: odd widths under the relaxed ADMM algorithms only.
 bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
                          const PottsStateV& a, const PottsStateV& b);
 // For odd widths, whether the tile kernel that would otherwise run (its
@@ -438,6 +441,13 @@ cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsState
                             const AdmmCoef& K, float cu_in, int iters,
                             const PottsRowsMaps& src_maps, int fused, int* err,
                             cudaStream_t st);
+
+// Certificates of the state of M into at most eval_blocks(H, W) partials
+// (cmf_potts_cert.cuh), finished by eval_tail; a bounded wait that runs out
+// sets *err.
+cudaError_t potts_cert(int storage, const PottsProblem& P, const PottsRowsMaps& M, bool aniso,
+                       bool dr, float tau, double* partials, const EvalTail& T, int* err,
+                       cudaStream_t st);
 
 // --- TMA-staged Potts ADMM (cmf_potts_tma.cu) ---
 struct PottsTmaMaps {

@@ -29,10 +29,24 @@ cudaError_t potts_rows_tile_step_bf16(const PottsProblem& P, const PottsStateV& 
                                       const PottsRowsMaps& M, int fused, int* err,
                                       cudaStream_t st);
 
+cudaError_t potts_cert_f32(const PottsProblem& P, const PottsRowsMaps& M, bool aniso, bool dr,
+                           float tau, double* partials, const EvalTail& T, int* err,
+                           cudaStream_t st);
+cudaError_t potts_cert_f16(const PottsProblem& P, const PottsRowsMaps& M, bool aniso, bool dr,
+                           float tau, double* partials, const EvalTail& T, int* err,
+                           cudaStream_t st);
+cudaError_t potts_cert_bf16(const PottsProblem& P, const PottsRowsMaps& M, bool aniso, bool dr,
+                            float tau, double* partials, const EvalTail& T, int* err,
+                            cudaStream_t st);
+
 bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
                          const PottsStateV& a, const PottsStateV& b) {
+    return !(P.g.W % 2 && (K.ty || K.cp)) && potts_rows_layout(P, storage, a, b);
+}
+
+bool potts_rows_layout(const PottsProblem& P, int storage, const PottsStateV& a,
+                       const PottsStateV& b) {
     const Grid& G = P.g;
-    if (G.W % 2 && (K.ty || K.cp)) return false;
     if (P.L > rows::kMaxLabels || cost_src(P) != kCostF32) return false;
     // the last pair of an odd width writes its first element alone, every
     // other one a pair at an even offset
@@ -91,6 +105,16 @@ cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsState
         case CMF_F32: return potts_rows_step_f32(P, b, aniso, K, cu_in, iters, M, err, st);
         case CMF_F16: return potts_rows_step_f16(P, b, aniso, K, cu_in, iters, M, err, st);
         default: return potts_rows_step_bf16(P, b, aniso, K, cu_in, iters, M, err, st);
+    }
+}
+
+cudaError_t potts_cert(int storage, const PottsProblem& P, const PottsRowsMaps& M, bool aniso,
+                       bool dr, float tau, double* partials, const EvalTail& T, int* err,
+                       cudaStream_t st) {
+    switch (storage) {
+        case CMF_F32: return potts_cert_f32(P, M, aniso, dr, tau, partials, T, err, st);
+        case CMF_F16: return potts_cert_f16(P, M, aniso, dr, tau, partials, T, err, st);
+        default: return potts_cert_bf16(P, M, aniso, dr, tau, partials, T, err, st);
     }
 }
 
