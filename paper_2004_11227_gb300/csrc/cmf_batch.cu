@@ -14,6 +14,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <functional>
+#include <initializer_list>
 #include <vector>
 
 #include "cmf_kernels.cuh"
@@ -26,8 +28,14 @@ constexpr size_t kAl = 256;
 inline size_t al(size_t x) { return (x + kAl - 1) / kAl * kAl; }
 
 struct BatchLayout {
-    size_t desc, tiles, items, partials, scal, ctl, states, total;
+    size_t desc, tiles, items, partials, scal, ctl, states, maps, total;
     int n_bin_tiles, n_potts_tiles, n_bin_ev, n_potts_ev, potts_rows, max_l, n_strip_items;
+    // instances on the single solves' kernels (chains of warps; labels side by
+    // side, classes of at most 4, 8 and 16 labels)
+    bool chains;
+    int n_maps, n_chain_items, chain_rows;
+    int n_rows_items;  // room for their items (at bands of at most 12 rows)
+    int rows_rows[3], rows_labels[3];
 };
 
 // Whether a Potts instance of a batch runs by warp strips (the ADMM family,
@@ -50,6 +58,46 @@ int strip_items(const cmf_instance& in, const cmf_params& p) {
     return strip_count(in) * ((in.H + R - 1) / R);
 }
 
+// Instances the single solves' kernels take, under the relaxed ADMM algorithms.
+bool relaxed_admm(const cmf_params& p) {
+    return p.algo == CMF_PADMM || p.algo == CMF_RPADMM_FG || p.algo == CMF_RPADMM_EB;
+}
+Grid grid_of(const cmf_instance& in) {
+    return Grid{in.H, in.W, in.pitch, (size_t)in.H * (size_t)in.pitch};
+}
+int rows_class(int L) { return L <= 4 ? 0 : (L <= 8 ? 1 : 2); }
+bool batch_side(const cmf_instance& in, const cmf_params& p) {
+    if (in.model != 1 || !relaxed_admm(p)) return false;
+    const PottsProblem P{in.d_cost, in.L, Alpha{in.d_alpha, in.alpha0}, grid_of(in), nullptr,
+                         nullptr};
+    const PottsStateV s{in.d_u, in.d_qx, in.d_qy, in.d_p, (float*)in.d_ps};
+    return potts_rows_layout(P, p.storage, s, s);
+}
+bool batch_chain(const cmf_instance& in, const cmf_params& p) {
+    if (in.model != 0 || !relaxed_admm(p)) return false;
+    const Grid G = grid_of(in);
+    const BinProblem P{in.d_cost, in.d_cost + G.plane, Alpha{in.d_alpha, in.alpha0}, G};
+    const BinStateV s{in.d_u, in.d_qx, in.d_qy, in.d_ps, in.d_p};
+    return binary_chain_eligible(P, p.storage, s, s, s);
+}
+constexpr int kSideCols = 56;  // columns a strip of the labels side by side advances
+// Band height for instances of a class that together have `rows` strip rows:
+// rounds of the blocks a GB300 holds, each costing the band and the rows that
+// fill and drain it; ties to lower bands (they spread a batch's last, small
+// instances wider).
+int band_rows(long long rows, long long resident, int fill, std::initializer_list<int> heights) {
+    int best = 0;
+    long long cost = -1;
+    for (int r : heights) {
+        const long long c = ((rows + r - 1) / r + resident - 1) / resident * (r + fill);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = r;
+        }
+    }
+    return best;
+}
+
 int potts_rows_for(int maxL) { return maxL <= 8 ? 4 : (maxL <= 16 ? 2 : 1); }
 
 size_t state_bytes(const cmf_instance& in, int storage) {
@@ -59,8 +107,28 @@ size_t state_bytes(const cmf_instance& in, int storage) {
     return al(plane * 4 * in.L) + 3 * al(plane * es * in.L) + al(plane * 4);  // p_s float32
 }
 
-BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p) {
+// chains: instances on the single solves' kernels where they are eligible
+// (they need room for their tensor maps).
+BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
+                         bool chains = true) {
     BatchLayout b{};
+    b.chains = chains;
+    long long side_rows[3] = {0, 0, 0}, chain_rows = 0;
+    for (int i = 0; chains && i < n; ++i) {
+        const cmf_instance& in = inst[i];
+        const int k = rows_class(in.L);
+        if (batch_side(in, p)) {
+            side_rows[k] += (long long)((in.W + kSideCols - 1) / kSideCols) * in.H;
+            if (in.L > b.rows_labels[k]) b.rows_labels[k] = in.L;
+        } else if (batch_chain(in, p)) {
+            chain_rows += (long long)((in.W + batch_chain_cols() - 1) / batch_chain_cols()) * in.H;
+        }
+    }
+    for (int k = 0; k < 3; ++k)
+        b.rows_rows[k] = p.batch_rows > 0 ? p.batch_rows
+                                          : band_rows(side_rows[k], 152 * (3 - k), 8,
+                                                      {12, 16, 24, 32, 48});
+    b.chain_rows = band_rows(chain_rows, 152 * 4, 14, {8, 16, 24, 32, 48, 64});
     int maxL = 2;
     for (int i = 0; i < n; ++i)
         if (inst[i].model == 1 && inst[i].L > maxL) maxL = inst[i].L;
@@ -73,11 +141,21 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p) {
         const int ntx = (in.W + 31) / 32;
         const int ev = ntx * ((in.H + 31) / 32);
         if (in.model == 0) {
-            b.n_bin_tiles += ntx * ((in.H + 31) / 32);
+            if (chains && batch_chain(in, p)) {
+                b.n_chain_items += (in.W + batch_chain_cols() - 1) / batch_chain_cols() *
+                                   ((in.H + b.chain_rows - 1) / b.chain_rows);
+                ++b.n_maps;
+            } else {
+                b.n_bin_tiles += ntx * ((in.H + 31) / 32);
+            }
             b.n_bin_ev += ev;
         } else {
-            const int ty = 8 * b.potts_rows;
-            if (batch_strip(in, p))
+            const int ty = 8 * b.potts_rows, k = rows_class(in.L);
+            if (chains && batch_side(in, p)) {
+                const int r = b.rows_rows[k] < 12 ? b.rows_rows[k] : 12;
+                b.n_rows_items += (in.W + kSideCols - 1) / kSideCols * ((in.H + r - 1) / r);
+                ++b.n_maps;
+            } else if (batch_strip(in, p))
                 b.n_strip_items += strip_items(in, p);
             else
                 b.n_potts_tiles += ntx * ((in.H + ty - 1) / ty);
@@ -90,7 +168,7 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p) {
     b.tiles = off;
     off += al(sizeof(int) * (size_t)(b.n_bin_tiles + b.n_potts_tiles + b.n_bin_ev + b.n_potts_ev + 4));
     b.items = off;
-    off += al(sizeof(int2) * (size_t)(b.n_strip_items + 1));
+    off += al(sizeof(int2) * (size_t)(b.n_strip_items + b.n_chain_items + b.n_rows_items + 1));
     b.partials = off;
     off += al(sizeof(double) * 3 * (size_t)(b.n_bin_ev + b.n_potts_ev + 1));
     b.scal = off;
@@ -99,6 +177,8 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p) {
     off += al(64);
     b.states = off;
     for (int i = 0; i < n; ++i) off += state_bytes(inst[i], p.storage);
+    b.maps = off;
+    off += al(sizeof(BatchMaps) * (size_t)b.n_maps);
     b.total = off;
     return b;
 }
@@ -106,6 +186,7 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p) {
 struct BatchCtl {
     int it;
     int stop;
+    int err;  // kErrWaitTimeout: a bounded device-side wait ran out
 };
 
 __global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl) {
@@ -237,7 +318,8 @@ extern "C" size_t cmf_batch_workspace_bytes(const cmf_instance* inst, int n, con
     if (!inst || n < 1 || !p || check_batch_params(p) != CMF_OK) return 0;
     for (int i = 0; i < n; ++i)
         if (check_instance(inst[i], *p) != CMF_OK) return 0;
-    return batch_layout(inst, n, *p).total;
+    const size_t a = batch_layout(inst, n, *p).total, b = batch_layout(inst, n, *p, false).total;
+    return a > b ? a : b;
 }
 
 extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_params* p,
@@ -248,7 +330,8 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     for (int i = 0; i < n; ++i)
         if ((s = check_instance(inst[i], *p)) != CMF_OK) return s;
     if ((uintptr_t)d_ws % kAl) return CMF_EINVAL;
-    const BatchLayout B = batch_layout(inst, n, *p);
+    BatchLayout B = batch_layout(inst, n, *p);
+    if (ws_bytes < B.total) B = batch_layout(inst, n, *p, false);  // without the tensor maps
     if (ws_bytes < B.total) return CMF_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)d_ws;
@@ -262,6 +345,8 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     // (instance, strip item) of the strip-eligible Potts instances, even and
     // odd widths apart (the odd ones run the kernel with the last-pair masks)
     std::vector<int2> sitems, oitems;
+    std::vector<int2> citems, ritems[3];  // chains; labels side by side, by class
+    std::vector<BatchMaps> maps;
     char* sbase = ws + B.states;
     const int pty = 8 * B.potts_rows;
     for (int i = 0; i < n; ++i) {
@@ -304,7 +389,19 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             D.bw.pt = b;
             D.tile_base = (int)tb.size();
             D.ev_tab = (int)eb.size();
-            for (int t = 0; t < ntx * ((in.H + 31) / 32); ++t) tb.push_back(i);
+            if (B.chains && batch_chain(in, *p)) {
+                D.sp_out = batch_chain_cols();
+                D.sp_nstrips = (in.W + D.sp_out - 1) / D.sp_out;
+                D.sp_rows = B.chain_rows;
+                D.maps = (int)maps.size();
+                maps.emplace_back();
+                CMF_CUDA_TRY(binary_chain_maps(D.bp, p->storage, D.bu, maps.back().set[0].binary));
+                CMF_CUDA_TRY(binary_chain_maps(D.bp, p->storage, D.bw, maps.back().set[1].binary));
+                for (int t = 0; t < D.sp_nstrips * ((in.H + D.sp_rows - 1) / D.sp_rows); ++t)
+                    citems.push_back(make_int2(i, t));
+            } else {
+                for (int t = 0; t < ntx * ((in.H + 31) / 32); ++t) tb.push_back(i);
+            }
             for (int t = 0; t < D.ev_count; ++t) eb.push_back(i);
         } else {
             D.pp = PottsProblem{in.d_cost, in.L, A, G, nullptr};
@@ -321,7 +418,19 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             D.pw.ps = (float*)b;
             D.tile_base = (int)tp.size();
             D.ev_tab = (int)ep.size();
-            if (batch_strip(in, *p)) {
+            if (B.chains && batch_side(in, *p)) {
+                const int k = rows_class(in.L);
+                D.sp_out = kSideCols;
+                D.sp_nstrips = (in.W + kSideCols - 1) / kSideCols;
+                D.sp_rows = B.rows_rows[k];
+                D.maps = (int)maps.size();
+                maps.emplace_back();
+                CMF_CUDA_TRY(potts_rows_maps(D.pp, p->storage, D.pu, maps.back().set[0].potts));
+                CMF_CUDA_TRY(potts_rows_maps(D.pp, p->storage, D.pw, maps.back().set[1].potts));
+                for (int t = 0; t < D.sp_nstrips * ((in.H + D.sp_rows - 1) / D.sp_rows); ++t)
+                    ritems[k].push_back(make_int2(i, t));
+            } else if (batch_strip(in, *p)) {
+                D.sp_out = 60;
                 D.sp_nstrips = strip_count(in);
                 D.sp_rows = strip_rows(*p);
                 std::vector<int2>& dst = in.W % 2 ? oitems : sitems;
@@ -353,14 +462,26 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     if (!all.empty())
         CMF_CUDA_TRY(cudaMemcpyAsync(tables, all.data(), sizeof(int) * all.size(),
                                      cudaMemcpyHostToDevice, st));
+    // one table after the other: the Potts items first (their finalize launch
+    // takes them all), then the chains'
+    std::vector<int2> table;
+    for (const std::vector<int2>* v : {&sitems, &oitems, &ritems[0], &ritems[1], &ritems[2], &citems})
+        table.insert(table.end(), v->begin(), v->end());
     int2* d_items = (int2*)(ws + B.items);
     int2* d_oitems = d_items + sitems.size();
-    if (!sitems.empty())
-        CMF_CUDA_TRY(cudaMemcpyAsync(d_items, sitems.data(), sizeof(int2) * sitems.size(),
+    int2* d_ritems[3];
+    d_ritems[0] = d_oitems + oitems.size();
+    d_ritems[1] = d_ritems[0] + ritems[0].size();
+    d_ritems[2] = d_ritems[1] + ritems[1].size();
+    int2* d_citems = d_ritems[2] + ritems[2].size();
+    if (!table.empty())
+        CMF_CUDA_TRY(cudaMemcpyAsync(d_items, table.data(), sizeof(int2) * table.size(),
                                      cudaMemcpyHostToDevice, st));
-    if (!oitems.empty())
-        CMF_CUDA_TRY(cudaMemcpyAsync(d_oitems, oitems.data(), sizeof(int2) * oitems.size(),
+    BatchMaps* d_maps = (BatchMaps*)(ws + B.maps);
+    if (!maps.empty())
+        CMF_CUDA_TRY(cudaMemcpyAsync(d_maps, maps.data(), sizeof(BatchMaps) * maps.size(),
                                      cudaMemcpyHostToDevice, st));
+    CMF_CUDA_TRY(cudaMemsetAsync(&ctl->err, 0, sizeof(int), st));
     // cold starts
     if (!p->warm_start) {
         for (int i = 0; i < n; ++i) {
@@ -374,29 +495,89 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     k_batch_reset<<<1, 256, 0, st>>>(d_desc, n, ctl);
     CMF_CUDA_TRY(cudaGetLastError());
 
-    // one chunk: check_every iterations of every active instance, the
-    // certificates and the per-instance stop decision
-    auto enqueue_chunk = [&](cudaStream_t s, cudaGraphConditionalHandle h,
-                             int set_h) -> cudaError_t {
-        cudaError_t e = cudaSuccess;
-        for (int k = 0; k < p->check_every && e == cudaSuccess; ++k) {
-            const int parity = k & 1;
-            if (!tb.empty())
+    // coefficients shared by the instances on the single solves' kernels (their
+    // kernels take 1 / a_2 from the instance)
+    const AdmmCoef Ks = make_admm_coef(*p, 2);
+    // The chunk's iterations as independent tracks (an instance belongs to one
+    // of them): launches of one track follow one another, tracks need not.
+    const int K = p->check_every;
+    std::vector<std::function<cudaError_t(cudaStream_t)>> tracks;
+    if (!tb.empty())
+        tracks.push_back([&](cudaStream_t s) {
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < K && e == cudaSuccess; ++k)
                 e = batch_binary_step(p->storage, aniso, dr, p->sweeps, d_desc, d_tb,
-                                      (int)tb.size(), parity, s);
-            if (e == cudaSuccess && !tp.empty())
+                                      (int)tb.size(), k & 1, s);
+            return e;
+        });
+    if (!tp.empty())
+        tracks.push_back([&](cudaStream_t s) {
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < K && e == cudaSuccess; ++k)
                 e = batch_potts_step(p->storage, aniso, dr, p->sweeps, B.potts_rows, B.max_l,
-                                     d_desc, d_tp, (int)tp.size(), parity, s);
-            if (e == cudaSuccess && !sitems.empty())
-                e = batch_potts_strip_step(p->storage, aniso, false, d_desc, d_items,
-                                           (int)sitems.size(), parity, k == 0, s);
-            if (e == cudaSuccess && !oitems.empty())
-                e = batch_potts_strip_step(p->storage, aniso, true, d_desc, d_oitems,
-                                           (int)oitems.size(), parity, k == 0, s);
+                                     d_desc, d_tp, (int)tp.size(), k & 1, s);
+            return e;
+        });
+    for (int odd = 0; odd < 2; ++odd)
+        if (!(odd ? oitems : sitems).empty())
+            tracks.push_back([&, odd](cudaStream_t s) {
+                cudaError_t e = cudaSuccess;
+                for (int k = 0; k < K && e == cudaSuccess; ++k)
+                    e = batch_potts_strip_step(p->storage, aniso, odd == 1, d_desc,
+                                               odd ? d_oitems : d_items,
+                                               (int)(odd ? oitems : sitems).size(), k & 1, k == 0,
+                                               s);
+                return e;
+            });
+    for (int c = 0; c < 3; ++c)
+        if (!ritems[c].empty())
+            tracks.push_back([&, c](cudaStream_t s) {
+                // pairs; two single iterations where that makes the launches
+                // even, so that the chunk ends in the callers' buffers
+                const int singles = (K / 2) % 2 ? 2 : 0;
+                cudaError_t e = cudaSuccess;
+                for (int k = 0, m = 0; k < K && e == cudaSuccess; ++m) {
+                    const int it = k < singles ? 1 : 2;
+                    e = batch_potts_rows_step(p->storage, aniso, 4 << c, B.rows_labels[c], it,
+                                              d_desc, d_maps, d_ritems[c], (int)ritems[c].size(),
+                                              Ks, m & 1, k == 0, &ctl->err, s);
+                    k += it;
+                }
+                return e;
+            });
+    if (!citems.empty())
+        tracks.push_back([&](cudaStream_t s) {
+            // an even number of launches of about equal length
+            const int most = binary_chain_max_iters(false);
+            const int nl = 2 * ((K + 2 * most - 1) / (2 * most));
+            cudaError_t e = cudaSuccess;
+            for (int m = 0; m < nl && e == cudaSuccess; ++m)
+                e = batch_binary_chain_step(p->storage, aniso, K / nl + (m < K % nl ? 1 : 0),
+                                            d_desc, d_maps, d_citems, (int)citems.size(), Ks,
+                                            m & 1, &ctl->err, s);
+            return e;
+        });
+    // one chunk: check_every iterations of every active instance, the
+    // certificates and the per-instance stop decision.  side: streams the
+    // tracks run beside the first one on (a graph being captured), or none.
+    auto enqueue_chunk = [&](cudaStream_t s, cudaGraphConditionalHandle h, int set_h,
+                             const std::vector<cudaStream_t>& side,
+                             const std::vector<cudaEvent_t>& ev) -> cudaError_t {
+        cudaError_t e = cudaSuccess;
+        for (size_t t = 1; t < tracks.size() && t <= side.size() && e == cudaSuccess; ++t) {
+            if (t == 1) e = cudaEventRecord(ev[0], s);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(side[t - 1], ev[0], 0);
+        }
+        for (size_t t = 0; t < tracks.size() && e == cudaSuccess; ++t)
+            e = tracks[t](t == 0 || side.empty() ? s : side[t - 1]);
+        for (size_t t = 1; t < tracks.size() && t <= side.size() && e == cudaSuccess; ++t) {
+            e = cudaEventRecord(ev[t], side[t - 1]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[t], 0);
         }
         // the strip instances hold w = u - cu p_s after the chunk: back to u
-        // (both tables are contiguous in the workspace)
-        const int nall = (int)(sitems.size() + oitems.size());
+        // (their tables are contiguous in the workspace)
+        const int nall = (int)(sitems.size() + oitems.size() + ritems[0].size() +
+                               ritems[1].size() + ritems[2].size());
         if (e == cudaSuccess && nall > 0)
             e = batch_potts_strip_finalize(d_desc, d_items, nall, s);
         if (e == cudaSuccess && !eb.empty())
@@ -414,6 +595,9 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         return e;
     };
     auto collect = [&]() -> cmf_status {
+        int herr = 0;
+        CMF_CUDA_TRY(cudaMemcpy(&herr, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost));
+        if (herr == kErrWaitTimeout) return CMF_ETIMEOUT;
         bool all_ok = true;
         for (int i = 0; i < n; ++i) {
             inst[i].iters = desc[i].iters;
@@ -429,7 +613,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     if (!p->use_graph) {
         // host-driven: one chunk per round trip, the stop flag read back
         for (;;) {
-            CMF_CUDA_TRY(enqueue_chunk(st, 0, 0));
+            CMF_CUDA_TRY(enqueue_chunk(st, 0, 0, {}, {}));
             BatchCtl hc;
             CMF_CUDA_TRY(cudaMemcpyAsync(&hc, ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
             CMF_CUDA_TRY(cudaStreamSynchronize(st));
@@ -442,11 +626,24 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     }
 
     cudaStream_t cs = nullptr;
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> ev;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ge = nullptr;
     cmf_status status = CMF_ECUDA;
     do {
         if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) break;
+        bool made = true;
+        for (size_t t = 0; t < tracks.size() && made; ++t) {
+            cudaEvent_t x = nullptr;
+            made = cudaEventCreateWithFlags(&x, cudaEventDisableTiming) == cudaSuccess;
+            if (made) ev.push_back(x);
+            cudaStream_t y = nullptr;
+            if (t == 0) continue;
+            made = made && cudaStreamCreateWithFlags(&y, cudaStreamNonBlocking) == cudaSuccess;
+            if (made) side.push_back(y);
+        }
+        if (!made) break;
         if (cudaGraphCreate(&g, 0) != cudaSuccess) break;
         cudaGraphConditionalHandle h;
         if (cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) !=
@@ -462,7 +659,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         if (cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                           cudaStreamCaptureModeRelaxed) != cudaSuccess)
             break;
-        const cudaError_t e = enqueue_chunk(cs, h, 1);
+        const cudaError_t e = enqueue_chunk(cs, h, 1, side, ev);
         cudaGraph_t captured = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
         if (e != cudaSuccess || e2 != cudaSuccess) break;
@@ -477,6 +674,8 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     if (ge) cudaGraphExecDestroy(ge);
     if (g) cudaGraphDestroy(g);
     if (cs) cudaStreamDestroy(cs);
+    for (cudaStream_t x : side) cudaStreamDestroy(x);
+    for (cudaEvent_t x : ev) cudaEventDestroy(x);
     return status;
 }
 
@@ -489,7 +688,7 @@ extern "C" cmf_status cmf_autotune_batch(cmf_instance* inst, int n, const cmf_pa
     bool strips = false;
     for (int i = 0; i < n; ++i) {
         if ((s = check_instance(inst[i], *p)) != CMF_OK) return s;
-        strips = strips || batch_strip(inst[i], *p);
+        strips = strips || batch_strip(inst[i], *p) || batch_side(inst[i], *p);
     }
     std::vector<cmf_params> cand;
     for (int f : {1, 2, 5}) {
@@ -506,7 +705,7 @@ extern "C" cmf_status cmf_autotune_batch(cmf_instance* inst, int n, const cmf_pa
     }
     cudaStream_t st = (cudaStream_t)stream;
     // one untimed solve first: module loading and first launches
-    if (!cand.empty() && batch_layout(inst, n, cand[0]).total <= ws_bytes) {
+    if (!cand.empty() && batch_layout(inst, n, cand[0], false).total <= ws_bytes) {
         s = cmf_solve_batch(inst, n, &cand[0], d_ws, ws_bytes, stream);
         if (s == CMF_ECUDA || s == CMF_ETIMEOUT || s == CMF_EINVAL) return s;
     }
@@ -517,7 +716,7 @@ extern "C" cmf_status cmf_autotune_batch(cmf_instance* inst, int n, const cmf_pa
     bool found = false;
     cmf_status last = CMF_NOT_CONVERGED;
     for (const cmf_params& q : cand) {
-        if (batch_layout(inst, n, q).total > ws_bytes) {
+        if (batch_layout(inst, n, q, false).total > ws_bytes) {
             last = CMF_ENOMEM;
             continue;
         }

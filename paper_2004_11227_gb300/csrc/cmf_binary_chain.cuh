@@ -160,11 +160,14 @@ __device__ __forceinline__ void project(float& x, float& y, float al, bool swap)
 // way round at odd columns, and with 16-bit flows the second iteration of
 // their pairs does at even ones too (iter0: the call's index of warp 0's
 // iteration).
+//
+// One block: the band r0 .. r1-1 of the strip whose first staged column is
+// cfirst (hl and hr: its halo columns), from the state of M into s1.
 template <typename S, bool ANISO, bool SIMPLE, bool EVEN, bool CERT>
-__global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMaxIters + 1), CERT ? 3 : 4)
-    k_binary_chain(const __grid_constant__ BinChainMaps M, BinProblem Pr, BinState<S> s1,
-                   AdmmCoef K, int T, int iter0, int R, int nstrips, double* partials,
-                   EvalTail tail, int* err) {
+__device__ __forceinline__ void binary_chain_block(
+    const BinChainMaps& M, const BinProblem& Pr, const BinState<S>& s1, const AdmmCoef& K,
+    const int T, const int iter0, const int r0, const int r1, const int cfirst, const int hl,
+    const int hr, DF& accE, DF& accD, DF& accR, int* err) {
     using namespace chain;
     using St = Store<S>;
     using QS = Quad<S>;
@@ -178,10 +181,6 @@ __global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMax
     const unsigned full_mask = 0xffffffffu;
     const int links = T - 1 + (CERT ? 1 : 0);  // handovers between warps
 
-    const int r0 = (blockIdx.x / nstrips) * R;
-    const int r1 = min(r0 + R, G.H);
-    const int hl = left_cols(T), hr = right_cols(T, CERT);
-    const int cfirst = (int)(blockIdx.x % nstrips) * (kCols - hl - hr) - hl;
     const int c = cfirst + 4 * lane;
     const bool own = 4 * lane >= hl && 4 * lane < kCols - hr && c < G.W;
     const int offs = cfirst & (Seg<ES>::align - 1);  // float32 segments start at cfirst
@@ -202,7 +201,6 @@ __global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMax
                 Pr.alpha.value;
     __syncthreads();
 
-    DF accE = {0.f, 0.f}, accD = {0.f, 0.f}, accR = {0.f, 0.f};
     if (wib == T + (CERT ? 2 : 0)) {
         // ---- producer ------------------------------------------------------
         const uint32_t tx = 4u * Seg<ES>::row + (has_al ? 4u : 3u) * Seg<4>::row;
@@ -509,6 +507,21 @@ __global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMax
             }
         }
     }
+}
+
+// One launch of the single-problem solver.
+template <typename S, bool ANISO, bool SIMPLE, bool EVEN, bool CERT>
+__global__ void __launch_bounds__(32 * (CERT ? chain::kMaxCert + 3 : chain::kMaxIters + 1), CERT ? 3 : 4)
+    k_binary_chain(const __grid_constant__ BinChainMaps M, BinProblem P, BinState<S> s1,
+                   AdmmCoef K, int T, int iter0, int R, int nstrips, double* partials,
+                   EvalTail tail, int* err) {
+    const int hl = chain::left_cols(T), hr = chain::right_cols(T, CERT);
+    const int r0 = (blockIdx.x / nstrips) * R;
+    DF accE = {0.f, 0.f}, accD = {0.f, 0.f}, accR = {0.f, 0.f};
+    binary_chain_block<S, ANISO, SIMPLE, EVEN, CERT>(
+        M, P, s1, K, T, iter0, r0, min(r0 + R, P.g.H),
+        (int)(blockIdx.x % nstrips) * (chain::kCols - hl - hr) - hl, hl, hr, accE, accD, accR,
+        err);
     if (CERT) {
         block_reduce3_store_df(accE, accD, accR, partials + 3 * (size_t)blockIdx.x);
         eval_tail(tail, partials, gridDim.x);

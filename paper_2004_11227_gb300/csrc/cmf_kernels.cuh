@@ -499,6 +499,16 @@ struct BatchDesc {
     DrCoef dk;
     int sp_nstrips;        // Potts by warp strips: strips of the grid (0: tiles)
     int sp_rows;           // band height of its strip items
+    int sp_out;            // columns a strip advances
+    int maps;              // index of its tensor map sets (chains, labels side by side), or -1
+};
+
+// Tensor maps of a batch instance: the caller's state and the workspace's.
+struct BatchMaps {
+    union {
+        PottsRowsMaps potts;
+        BinChainMaps binary;
+    } set[2];
 };
 
 // parity 0: caller's buffers -> workspace; 1: workspace -> caller's buffers
@@ -518,6 +528,20 @@ cudaError_t batch_potts_strip_step(int storage, bool aniso, bool odd_width, cons
 cudaError_t batch_potts_strip_finalize(const BatchDesc* desc, const int2* items, int nitems,
                                        cudaStream_t st);
 int potts_strip_max_rows();  // band rows the strip kernels take at most
+
+// Potts instances of at most lc labels (4, 8 or 16) with the labels side by
+// side: `iters` (1 or 2) iterations over a table of (instance, item) pairs;
+// nlab: the most labels among them, K: the coefficients but for a_2.
+cudaError_t batch_potts_rows_step(int storage, bool aniso, int lc, int nlab, int iters,
+                                  const BatchDesc* desc, const BatchMaps* maps, const int2* items,
+                                  int nitems, const AdmmCoef& K, int parity, int first, int* err,
+                                  cudaStream_t st);
+// Binary instances by chains of warps: T iterations (strips of
+// batch_chain_cols() columns).
+cudaError_t batch_binary_chain_step(int storage, bool aniso, int T, const BatchDesc* desc,
+                                    const BatchMaps* maps, const int2* items, int nitems,
+                                    const AdmmCoef& K, int parity, int* err, cudaStream_t st);
+int batch_chain_cols();
 
 cudaError_t batch_binary_eval(int storage, bool aniso, bool dr, float tau,
                               const BatchDesc* desc, const int* tile_inst, int ntiles,

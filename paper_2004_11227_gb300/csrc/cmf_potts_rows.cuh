@@ -173,18 +173,20 @@ struct Row {
 // solve's p_s keeps a rounding difference of single iterations (its weakly
 // determined directions hardly contract), so the results of a problem do not
 // depend on which kernel ran it.  fused (TILE): products rounded into the sums.
+//
+// One block: the band r0 .. r1-1 of the strip whose first staged column is
+// cfirst, from the state of M into s1.
 template <typename S, bool ANISO, bool SIMPLE, int T, int LC, bool TILE>
-__global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
-                                  LC == 4 ? 4 : (LC == 8 ? 2 : 1))
-    k_potts_rows(const __grid_constant__ PottsRowsMaps M, PottsProblem P, PottsState<S> s1,
-                 AdmmCoef K, float cu_in, int R, int nstrips, int fused, int* err) {
+__device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const PottsProblem& P,
+                                                 const PottsState<S>& s1, const AdmmCoef& K,
+                                                 const float cu_in, const int r0, const int r1,
+                                                 const int cfirst, const int fused, int* err) {
     using namespace rows;
     using St = Store<S>;
     using PS = Pair<S>;
     constexpr int ES = sizeof(S);
     using Y = Layout<LC, ES, TILE>;
-    constexpr int OUT = T == 2 ? 56 : 60;  // owned columns
-    constexpr int HL = T == 2 ? 2 : 1;     // halo lanes on each side
+    constexpr int HL = T == 2 ? 2 : 1;  // halo lanes on each side
     extern __shared__ __align__(128) unsigned char dsm_raw[];
     const Grid G = P.g;
     const int L = P.L;
@@ -194,9 +196,6 @@ __global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned full_mask = 0xffffffffu;
 
-    const int r0 = (blockIdx.x / nstrips) * R;
-    const int r1 = min(r0 + R, G.H);
-    const int cfirst = (int)(blockIdx.x % nstrips) * OUT - 2 * HL;
     const int c = cfirst + 2 * lane;
     const bool own = lane >= HL && lane <= 31 - HL && c < G.W;
     const bool pair = c + 1 < G.W;  // else the last column of an odd width alone
@@ -236,6 +235,7 @@ __global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
     if (wib >= L) {
         // ---- service warps: the label sums; the input rows -------------------
         constexpr bool two = service_warps(T, LC) == 2;
+        if (wib >= L + service_warps(T, LC)) return;  // a block sized for more labels
         const bool sums = !two || wib == L, inputs = !two || wib > L;
         const uint32_t tx = (uint32_t)L * (3u * Seg<ES>::cols * ES + 2u * Seg<4>::cols * 4u) +
                             (has_al ? 2u : 1u) * Seg<4>::cols * 4u;
@@ -525,6 +525,18 @@ __global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
         }
     }
     if (!ok && lane == 0) atomicExch(err, kErrWaitTimeout);
+}
+
+// One launch of the single-problem solver.
+template <typename S, bool ANISO, bool SIMPLE, int T, int LC, bool TILE>
+__global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
+                                  LC == 4 ? 4 : (LC == 8 ? 2 : 1))
+    k_potts_rows(const __grid_constant__ PottsRowsMaps M, PottsProblem P, PottsState<S> s1,
+                 AdmmCoef K, float cu_in, int R, int nstrips, int fused, int* err) {
+    const int r0 = (blockIdx.x / nstrips) * R;
+    potts_rows_block<S, ANISO, SIMPLE, T, LC, TILE>(
+        M, P, s1, K, cu_in, r0, min(r0 + R, P.g.H),
+        (int)(blockIdx.x % nstrips) * (T == 2 ? 56 : 60) - (T == 2 ? 4 : 2), fused, err);
 }
 
 // ---- host side -------------------------------------------------------------

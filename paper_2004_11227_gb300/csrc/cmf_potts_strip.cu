@@ -312,11 +312,10 @@ __global__ void k_batch_potts_strip_finalize(const BatchDesc* __restrict__ desc,
         const BatchDesc* D = desc + e.x;
         if (!D->active) continue;
         const Grid G = D->pp.g;
-        const int cs = (e.y % D->sp_nstrips) * kStripOut;
         const int r0 = (e.y / D->sp_nstrips) * D->sp_rows;
         const int r1 = min(r0 + D->sp_rows, G.H);
-        const int c = cs - 2 + 2 * lane;
-        if (lane < 1 || lane > 30 || c >= G.W) continue;
+        const int c = (e.y % D->sp_nstrips) * D->sp_out + 2 * lane;
+        if (2 * lane >= D->sp_out || c >= G.W) continue;
         const float cu = D->ak.cu;
         float* u = D->pu.u;
         const float* ps = D->pu.ps;
