@@ -352,17 +352,30 @@ def cmf_eval_binary_noalloc(b: Binary, stream=None):
     return tuple(out)
 
 
+def _history(hist_cap: int):
+    """A history array.  Up to 65536 rows the number a solve writes follows
+    from its iterations (``_rows``) and the array needs no zeros."""
+    return np.empty((hist_cap, 5)) if hist_cap <= 65536 else np.zeros((hist_cap, 5))
+
+
+def _rows(hist, p: Params, iters: int):
+    """The rows a solve has written: one per check, every check_every
+    iterations and at the last one."""
+    cap = len(hist)
+    return hist[:min(-(-iters // p.check_every), cap) if cap <= 65536
+                else int(np.count_nonzero(hist[:, 0]))]
+
+
 def cmf_solve_binary(b: Binary, hist_cap: int = 4096, stream=None):
     """Returns (status, iterations, history array [n, 5])."""
-    hist = np.zeros((hist_cap, 5))
+    hist = _history(hist_cap)
     iters = ctypes.c_int(0)
     st = _check(lib().cmf_solve_binary(*b._common(), *b._state_ptrs(),
                                        hist.ctypes.data_as(ctypes.c_void_p), hist_cap,
                                        ctypes.byref(iters), _ptr(b.ws), b.ws.numel(),
                                        _stream(stream)),
                 "cmf_solve_binary", allow=(OK, NOT_CONVERGED))
-    n = int(np.count_nonzero(hist[:, 0]))
-    return st, iters.value, hist[:n]
+    return st, iters.value, _rows(hist, b.params, iters.value)
 
 
 def cmf_init_potts(s: Potts, stream=None) -> None:
@@ -383,15 +396,14 @@ def cmf_eval_potts(s: Potts, stream=None):
 
 
 def cmf_solve_potts(s: Potts, hist_cap: int = 4096, stream=None):
-    hist = np.zeros((hist_cap, 5))
+    hist = _history(hist_cap)
     iters = ctypes.c_int(0)
     st = _check(lib().cmf_solve_potts(*s._common(), *s._state_ptrs(),
                                       hist.ctypes.data_as(ctypes.c_void_p), hist_cap,
                                       ctypes.byref(iters), _ptr(s.ws), s.ws.numel(),
                                       _stream(stream)),
                 "cmf_solve_potts", allow=(OK, NOT_CONVERGED))
-    n = int(np.count_nonzero(hist[:, 0]))
-    return st, iters.value, hist[:n]
+    return st, iters.value, _rows(hist, s.params, iters.value)
 
 
 class Batch:

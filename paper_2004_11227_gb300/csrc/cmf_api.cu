@@ -705,6 +705,7 @@ __global__ void k_solve_reset(SolveCtl* ctl, int it0) {
     ctl->stop = 0;
     ctl->where = 0;
     ctl->arrive = 0;
+    ctl->err = 0;  // an earlier phase's error was reported with its last certificates
 }
 
 // End of a two-chunk loop body: go on unless either half stopped.
@@ -724,6 +725,13 @@ bool graph_eligible(const cmf_params& p) {
     if (!p.use_graph || p.max_iter < p.check_every) return false;
     if (p.max_iter % p.check_every != 0) return false;
     return true;
+}
+
+// The error word at the start of a solve: the loop's reset kernel clears it,
+// unless iterations run host-driven before it.
+cudaError_t clear_error(const cmf_params& p, int* err, cudaStream_t st) {
+    if (graph_eligible(p) && p.rho_schedule_len == 0) return cudaSuccess;
+    return cudaMemsetAsync(err, 0, sizeof(int), st);
 }
 
 // Everything the kernels of a solve graph are built from: the device, the
@@ -966,15 +974,28 @@ cmf_status solve_graph(const cmf_params* p, const SolveSig& sig, char* wsbase, c
         graph_drop(ge);
         return CMF_ECUDA;
     }
-    SolveCtl hc;
-    CMF_CUDA_TRY(cudaMemcpyAsync(&hc, ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
-    CMF_CUDA_TRY(cudaStreamSynchronize(st));
-    const int n = hc.checks < rows ? hc.checks : rows;
+    // The control block and the first history rows follow one another in the
+    // workspace: one copy brings both home (a copy and its synchronisation cost
+    // about 10 us, a 64^2 solve 150), a second one only rows beyond them.
     const int room = hist_cap > nh0 ? hist_cap - nh0 : 0;
-    const int ncopy = n < room ? n : room;
-    if (h_hist && ncopy > 0)
-        CMF_CUDA_TRY(cudaMemcpy(h_hist + 5 * (size_t)nh0, dhist, sizeof(double) * 5 * (size_t)ncopy,
-                                cudaMemcpyDeviceToHost));
+    const int want = h_hist ? (rows < room ? rows : room) : 0;
+    constexpr int kFirstRows = 96;
+    const int head = want < kFirstRows ? want : kFirstRows;
+    const size_t row_bytes = 5 * sizeof(double), hist_at = w.hist - w.ctl;
+    double buf[(256 + kFirstRows * 5 * sizeof(double)) / sizeof(double)];
+    static_assert(sizeof(SolveCtl) <= 256, "the history follows the control block's 256 bytes");
+    CMF_CUDA_TRY(cudaMemcpyAsync(buf, ctl, head > 0 ? hist_at + head * row_bytes : sizeof(SolveCtl),
+                                 cudaMemcpyDeviceToHost, st));
+    CMF_CUDA_TRY(cudaStreamSynchronize(st));
+    SolveCtl hc;
+    memcpy(&hc, buf, sizeof(hc));
+    const int n = hc.checks < want ? hc.checks : want;
+    if (n > 0)
+        memcpy(h_hist + 5 * (size_t)nh0, (const char*)buf + hist_at,
+               (n < head ? n : head) * row_bytes);
+    if (n > head)
+        CMF_CUDA_TRY(cudaMemcpy(h_hist + 5 * (size_t)(nh0 + head), dhist + 5 * (size_t)head,
+                                (n - head) * row_bytes, cudaMemcpyDeviceToHost));
     if (h_iters) *h_iters = hc.it;
     if (hc.where != 0) {  // stopped after the first half of a two-chunk body
         CMF_CUDA_TRY(copy_back(hc.where));
@@ -1181,7 +1202,7 @@ cmf_status cmf_solve_binary(const float* d_Cs, const float* d_Ct, const float* d
     if (s != CMF_OK) return s;
     if (hist_cap < 0) return CMF_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    CMF_CUDA_TRY(cudaMemsetAsync(&((SolveCtl*)(c.wsbase + c.w.ctl))->err, 0, sizeof(int), st));
+    CMF_CUDA_TRY(clear_error(*p, c.err, st));
     if (!p->warm_start)
         CMF_CUDA_TRY(binary_init(c.storage, c.P, c.user, c.cfg.dr, c.cfg.dc.tau, st));
     const SolveSig sig = make_sig(0, 2, H, W, pitch, alpha0,
@@ -1283,7 +1304,7 @@ cmf_status cmf_solve_potts(const float* d_C, int L, const float* d_alpha, float 
     if (s != CMF_OK) return s;
     if (hist_cap < 0) return CMF_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    CMF_CUDA_TRY(cudaMemsetAsync(c.err, 0, sizeof(int), st));
+    CMF_CUDA_TRY(clear_error(*p, c.err, st));
     int it0 = 0, nh0 = 0;
     if (p->phase_storage != 0) {
         // phase one: the same solve in 16-bit flow storage, in the
