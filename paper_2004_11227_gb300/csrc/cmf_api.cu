@@ -516,6 +516,7 @@ struct PottsCall {
     bool strip;                  // fused ADMM by warp strips
     bool rows;                   // fused ADMM, labels side by side, up to two iterations a launch
     bool cert;                   // certificates with the labels side by side
+    bool dr_rows;                // rPDRQ with the labels side by side
     PottsTmaMaps maps[2];        // tensor maps of the user / workspace state sets
     PottsRowsMaps rmaps[2];
     int rfused;                  // potts_rows_fused
@@ -553,6 +554,7 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     call.tma = false;
     call.strip = false;
     call.rows = false;
+    call.dr_rows = false;
     // automatic choice: labels side by side (two iterations a launch; against
     // the strips 150 -> 64 us per iteration at 2048^2, L = 4 and 2293 -> 968 us
     // at 4096^2, L = 16, faster at every size measured from 128^2 and L = 2 on,
@@ -561,6 +563,11 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     call.cert = potts_rows_layout(call.P, p->storage, call.user, call.ws) &&
                 potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
                 potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess;
+    if (!call.cfg.plain && call.cfg.dr && p->variant == 0 && call.cert &&
+        potts_dr_rows_takes(call.P, call.cfg.dc)) {
+        call.dr_rows = true;
+        return CMF_OK;
+    }
     if (!call.cfg.plain && !call.cfg.dr && p->variant == 0 && call.cert &&
         potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws)) {
         call.rows = true;
@@ -649,6 +656,11 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
             cudaError_t e = potts_step(c.storage, c.P, c.user, c.user, cfg, tmp, st);
             if (e != cudaSuccess) return e;
             cur = 0;
+        } else if (c.dr_rows) {
+            cudaError_t e = potts_dr_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user,
+                                               cfg.aniso, cfg.dc, c.rmaps[cur], c.err, st);
+            if (e != cudaSuccess) return e;
+            cur ^= 1;
         } else if (c.strip && cfg.dr) {
             const PottsStateV& a = cur == 0 ? c.user : c.ws;
             const PottsStateV& b = cur == 0 ? c.ws : c.user;

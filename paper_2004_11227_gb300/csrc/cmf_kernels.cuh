@@ -442,6 +442,12 @@ cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsState
                             const PottsRowsMaps& src_maps, int fused, int* err,
                             cudaStream_t st);
 
+// One rPDRQ iteration from the state of src_maps into b (cmf_potts_dr_rows.cuh);
+// takes: whether the kernel does (beside potts_rows_layout).
+bool potts_dr_rows_takes(const PottsProblem& P, const DrCoef& D);
+cudaError_t potts_dr_rows_step(int storage, const PottsProblem& P, const PottsStateV& b,
+                               bool aniso, const DrCoef& D, const PottsRowsMaps& src_maps,
+                               int* err, cudaStream_t st);
 // Certificates of the state of M into at most eval_blocks(H, W) partials
 // (cmf_potts_cert.cuh), finished by eval_tail; a bounded wait that runs out
 // sets *err.

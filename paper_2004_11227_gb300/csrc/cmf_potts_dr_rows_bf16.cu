@@ -1,0 +1,11 @@
+// Potts rPDRQ with the labels side by side: __nv_bfloat16 flows.
+#include "cmf_potts_dr_rows.cuh"
+
+namespace cmf {
+
+cudaError_t potts_dr_rows_bf16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                               const DrCoef& D, const PottsRowsMaps& M, int* err, cudaStream_t st) {
+    return potts_dr_rows_s<__nv_bfloat16>(P, b, aniso, D, M, err, st);
+}
+
+}  // namespace cmf

@@ -1,0 +1,11 @@
+// Potts rPDRQ with the labels side by side: float flows.
+#include "cmf_potts_dr_rows.cuh"
+
+namespace cmf {
+
+cudaError_t potts_dr_rows_f32(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                              const DrCoef& D, const PottsRowsMaps& M, int* err, cudaStream_t st) {
+    return potts_dr_rows_s<float>(P, b, aniso, D, M, err, st);
+}
+
+}  // namespace cmf

@@ -39,6 +39,13 @@ cudaError_t potts_cert_bf16(const PottsProblem& P, const PottsRowsMaps& M, bool 
                             float tau, double* partials, const EvalTail& T, int* err,
                             cudaStream_t st);
 
+cudaError_t potts_dr_rows_f32(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                              const DrCoef& D, const PottsRowsMaps& M, int* err, cudaStream_t st);
+cudaError_t potts_dr_rows_f16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                              const DrCoef& D, const PottsRowsMaps& M, int* err, cudaStream_t st);
+cudaError_t potts_dr_rows_bf16(const PottsProblem& P, const PottsStateV& b, bool aniso,
+                               const DrCoef& D, const PottsRowsMaps& M, int* err, cudaStream_t st);
+
 bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
                          const PottsStateV& a, const PottsStateV& b) {
     return !(P.g.W % 2 && (K.ty || K.cp)) && potts_rows_layout(P, storage, a, b);
@@ -115,6 +122,24 @@ cudaError_t potts_cert(int storage, const PottsProblem& P, const PottsRowsMaps& 
         case CMF_F32: return potts_cert_f32(P, M, aniso, dr, tau, partials, T, err, st);
         case CMF_F16: return potts_cert_f16(P, M, aniso, dr, tau, partials, T, err, st);
         default: return potts_cert_bf16(P, M, aniso, dr, tau, partials, T, err, st);
+    }
+}
+
+bool potts_dr_rows_takes(const PottsProblem& P, const DrCoef& D) {
+    // one sweep, two columns per lane.  Against the strips faster at every size
+    // measured, 128^2 to 2048^2 and L = 2 to 16 (L = 2, 1024^2 51 -> 28 us;
+    // L = 4, 512^2 22.6 -> 16.5; L = 16, 2048^2 759 -> 520), with the same
+    // results; more labels, more sweeps and odd widths stay where they were.
+    return D.sweeps == 1 && P.g.W % 2 == 0;
+}
+
+cudaError_t potts_dr_rows_step(int storage, const PottsProblem& P, const PottsStateV& b,
+                               bool aniso, const DrCoef& D, const PottsRowsMaps& M, int* err,
+                               cudaStream_t st) {
+    switch (storage) {
+        case CMF_F32: return potts_dr_rows_f32(P, b, aniso, D, M, err, st);
+        case CMF_F16: return potts_dr_rows_f16(P, b, aniso, D, M, err, st);
+        default: return potts_dr_rows_bf16(P, b, aniso, D, M, err, st);
     }
 }
 
