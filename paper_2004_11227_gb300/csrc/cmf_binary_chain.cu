@@ -41,9 +41,15 @@ bool binary_chain_certifies(const Grid& G, int max_blocks) {
 
 cudaError_t binary_chain_maps(const BinProblem& P, int storage, const BinStateV& s,
                               BinChainMaps& m) {
+    return binary_row_maps(
+        P, storage, s, dtype_size(storage) == 4 ? chain::Seg<4>::cols : chain::Seg<2>::cols,
+        chain::Seg<4>::cols, m);
+}
+
+cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s, int cs, int c4,
+                            BinChainMaps& m) {
     const Grid& G = P.g;
     const int es = (int)dtype_size(storage);
-    const int cs = es == 4 ? chain::Seg<4>::cols : chain::Seg<2>::cols, c4 = chain::Seg<4>::cols;
     const struct {
         CUtensorMap* map;
         const void* base;

@@ -250,14 +250,25 @@ struct DrCoef {
 // q = qbar - tau grad u, p_t = pbar_t + tau u, p_s = pbar_s - tau u, then
 // qbar += rho (P_alpha(2q - qbar) - q), pbar_t += rho (min(2p_t - pbar_t, C_t)
 // - p_t), pbar_s += rho (min(2p_s - pbar_s + tau, C_s) - p_s).
-template <typename S, bool ANISO>
+// SWAP: the squares of the projection are added the other way round.
+template <typename S, bool ANISO, bool SWAP = false>
 __device__ __forceinline__ void binary_dr_flows(const DrCoef& D, float uc, float gx, float gy,
                                                 float qbx, float qby, float pbs, float pbt,
                                                 float al, float cs, float ct, float& oqx,
                                                 float& oqy, float& ops, float& opt) {
     const float q1 = qbx - D.tau * gx, q2 = qby - D.tau * gy;
     float tx = 2.f * q1 - qbx, ty = 2.f * q2 - qby;
-    project_alpha<ANISO>(tx, ty, al);
+    if (SWAP && !ANISO) {
+        al = fmaxf(al, 0.0f);
+        const float n2 = __fmaf_rn(ty, ty, __fmul_rn(tx, tx));
+        if (n2 > al * al) {
+            const float f = al * rsqrtf(n2);
+            tx *= f;
+            ty *= f;
+        }
+    } else {
+        project_alpha<ANISO>(tx, ty, al);
+    }
     oqx = qbx + D.rho * (tx - q1);
     oqy = qby + D.rho * (ty - q2);
     const float pt1 = pbt + D.tau * uc, ps1 = pbs - D.tau * uc;

@@ -392,6 +392,22 @@ cudaError_t binary_chain_step(
     int iter0, const BinChainMaps& src_maps, double* partials, int max_blocks, const EvalTail* cert, int* err,
     cudaStream_t st);
 
+// Maps of a state and its cost planes in boxes of one row: cs columns of the
+// stored flows, c4 of the float32 planes.
+cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s, int cs, int c4,
+                            BinChainMaps& m);
+
+// --- binary rPDRQ on warp-private TMA rings (cmf_binary_dr_rows.cu) ---
+// One iteration from the state of src_maps into b; a bounded wait that runs out
+// sets *err.
+bool binary_dr_rows_eligible(const BinProblem& P, int storage, const DrCoef& D,
+                             const BinStateV& a, const BinStateV& b);
+cudaError_t binary_dr_rows_maps(const BinProblem& P, int storage, const BinStateV& s,
+                                BinChainMaps& m);
+cudaError_t binary_dr_rows_step(int storage, const BinProblem& P, const BinStateV& b, bool aniso,
+                                const DrCoef& D, const BinChainMaps& src_maps, int* err,
+                                cudaStream_t st);
+
 // --- warp-strip Potts ADMM (cmf_potts_strip.cu) ---
 // Eligible: even W and pitch, H * pitch within int, pair-aligned planes.
 // odd_width_ok: the ADMM items of a batch also take odd widths (their last
