@@ -575,7 +575,7 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     call.rows = false;
     call.dr_rows = false;
     // automatic choice: labels side by side (two iterations a launch; against
-    // the strips 150 -> 64 us per iteration at 2048^2, L = 4 and 2293 -> 968 us
+    // the strips 150 -> 61.5 us per iteration at 2048^2, L = 4 and 2293 -> 937 us
     // at 4096^2, L = 16, faster at every size measured from 128^2 and L = 2 on,
     // with the same results), else warp strips where the layout allows them,
     // else TMA tiles, else shared-memory tiles

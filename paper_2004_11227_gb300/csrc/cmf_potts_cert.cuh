@@ -253,19 +253,19 @@ __global__ void __launch_bounds__(32 * (LC + cert::theta_warps(LC) + 1),
         const uint32_t tx = (uint32_t)L * (3u * Seg<ES>::cols * ES + 2u * Seg<4>::cols * 4u) +
                             (has_al ? 2u : 1u) * Seg<4>::cols * 4u;
         const int x4 = cfirst - off4, xs = cfirst - offs;
+        // one map a lane (q_x, q_y, p, u, p_s, C, alpha): its box, its slot's offset
+        const int nmaps = has_al ? 7 : 6;
+        const CUtensorMap* const map = &M.qx + (lane < nmaps ? lane : 0);
+        const int mx = lane < 3 ? xs : x4;
+        const int moff = lane < 4 ? lane * Y::fs
+                                  : Y::o_aux + (lane == 5 ? 0 : Y::f4 + (lane == 6 ? Y::f1 : 0));
         auto issue = [&](int i) {
-            if (i > il || lane != 0) return;
+            if (i > il) return;
             uint64_t* fb = bar + slot(i);
-            unsigned char* d = dsm + slot(i) * Y::state;
-            unsigned char* a = dsm + Y::o_aux + slot(i) * Y::aux;
-            mbar_arrive_expect_tx(fb, tx);
-            tma_load_3d(d, &M.qx, fb, xs, rf + i, 0);
-            tma_load_3d(d + Y::fs, &M.qy, fb, xs, rf + i, 0);
-            tma_load_3d(d + 2 * Y::fs, &M.p, fb, xs, rf + i, 0);
-            tma_load_3d(d + 3 * Y::fs, &M.u, fb, x4, rf + i, 0);
-            tma_load_3d(a, &M.C, fb, x4, rf + i, 0);
-            tma_load_3d(a + Y::f4, &M.ps, fb, x4, rf + i, 0);
-            if (has_al) tma_load_3d(a + Y::f4 + Y::f1, &M.al, fb, x4, rf + i, 0);
+            if (lane == 0) mbar_arrive_expect_tx(fb, tx);
+            __syncwarp();
+            unsigned char* d = dsm + moff + (lane < 4 ? slot(i) * Y::state : slot(i) * Y::aux);
+            if (lane < nmaps) tma_load_3d(d, map, fb, mx, rf + i, 0);
         };
         for (int i = 0; i < kRing; ++i) issue(i);
         int k = 0;

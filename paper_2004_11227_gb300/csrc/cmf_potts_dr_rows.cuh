@@ -29,7 +29,7 @@
 // blocks of 5 warps or two of 9 share an SM (rings of eight rows: 133 us, and
 // 105 at L = 8, 1024^2), and the label sums three rows ahead (two: 121 us).
 // Measured per iteration (CUDA events), one-label strips before: 2048^2 L = 4
-// float32 209 -> 117 us; 2048^2 L = 16 759 -> 520; 1024^2 L = 8 118 -> 70;
+// float32 209 -> 115 us; 1024^2 L = 16 227 -> 133; 1024^2 L = 8 118 -> 66;
 // 512^2 L = 4 22.6 -> 16.5; 128^2 L = 16 56 -> 12.4 (there a block is one
 // strip, and its labels no longer follow one another).  Same results bit for bit.
 #pragma once
@@ -117,19 +117,21 @@ __global__ void __launch_bounds__(32 * (LC + 1), LC == 4 ? 4 : (LC == 8 ? 2 : 1)
         const uint32_t tx = (uint32_t)L * (3u * Seg<ES>::cols * ES + 2u * Seg<4>::cols * 4u) +
                             (has_al ? 2u : 1u) * Seg<4>::cols * 4u;
         const int xs = cfirst - offs;
+        // one map a lane (q_x, q_y, p, u, p_s, C, alpha): its box, its slot's
+        // offset (one lane for all: 2048^2, L = 4 117 us, 1024^2, L = 8 70)
+        const int nmaps = has_al ? 7 : 6;
+        const CUtensorMap* const map = &M.qx + (lane < nmaps ? lane : 0);
+        const int mx = lane < 3 ? xs : cfirst;
+        const int moff = lane < 4 ? lane * Y::fs
+                                  : Y::o_aux + (lane == 5 ? 0 : Y::f4 + (lane == 6 ? Y::f1 : 0));
         auto issue = [&](int i) {
-            if (i > il || lane != 0) return;
+            if (i > il) return;
             uint64_t* fb = bar + (i & (kRing - 1));
-            unsigned char* d = dsm + (i & (kRing - 1)) * Y::state;
-            unsigned char* a = dsm + Y::o_aux + (i & (kAux - 1)) * Y::aux;
-            mbar_arrive_expect_tx(fb, tx);
-            tma_load_3d(d, &M.qx, fb, xs, rf + i, 0);
-            tma_load_3d(d + Y::fs, &M.qy, fb, xs, rf + i, 0);
-            tma_load_3d(d + 2 * Y::fs, &M.p, fb, xs, rf + i, 0);
-            tma_load_3d(d + 3 * Y::fs, &M.u, fb, cfirst, rf + i, 0);
-            tma_load_3d(a, &M.C, fb, cfirst, rf + i, 0);
-            tma_load_3d(a + Y::f4, &M.ps, fb, cfirst, rf + i, 0);
-            if (has_al) tma_load_3d(a + Y::f4 + Y::f1, &M.al, fb, cfirst, rf + i, 0);
+            if (lane == 0) mbar_arrive_expect_tx(fb, tx);
+            __syncwarp();
+            unsigned char* d =
+                dsm + moff + (lane < 4 ? (i & (kRing - 1)) * Y::state : (i & (kAux - 1)) * Y::aux);
+            if (lane < nmaps) tma_load_3d(d, map, fb, mx, rf + i, 0);
         };
         // sum over the labels, in label order, of float2s `stride` bytes apart
         auto label_sum = [&](const unsigned char* q, int stride) {

@@ -40,8 +40,8 @@
 // positions are constants (the row loop is unrolled by their length, eight),
 // 32-bit output indexes, and stage B before stage A rather than interleaved
 // (which spilled).  Measured per iteration (CUDA events), one-label strips
-// (odd widths: TMA tiles) before: 4096^2 L = 16 float32 2293 -> 968 us,
-// float16 1618 -> 971 us; 2048^2 L = 4 float32 150 -> 64 us; 512^2 L = 4
+// (odd widths: TMA tiles) before: 4096^2 L = 16 float32 2293 -> 937 us,
+// float16 1618 -> 964 us; 2048^2 L = 4 float32 150 -> 61.5 us; 512^2 L = 4
 // 26.8 -> 8.4 us; 721 x 1283, L = 8 94 -> 28 us.
 #pragma once
 
@@ -240,19 +240,23 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
         const uint32_t tx = (uint32_t)L * (3u * Seg<ES>::cols * ES + 2u * Seg<4>::cols * 4u) +
                             (has_al ? 2u : 1u) * Seg<4>::cols * 4u;
         const int x4 = cfirst - off4, xs = cfirst - offs;
+        // one map a lane (q_x, q_y, p, u, p_s, C, alpha): its box, its slot's
+        // offset (one lane issuing a row's seven boxes held the rows up: 2048^2,
+        // L = 4 float32 63.5 -> 61.5 us, float16 69.6 -> 63.9; 4096^2, L = 16
+        // 975 -> 937)
+        const int nmaps = has_al ? 7 : 6;
+        const CUtensorMap* const map = &M.qx + (lane < nmaps ? lane : 0);
+        const int mx = lane < 3 ? xs : x4;
+        const int moff = lane < 4 ? lane * Y::fs
+                                  : Y::o_aux + (lane == 5 ? 0 : Y::f4 + (lane == 6 ? Y::f1 : 0));
         auto issue = [&](int i) {
-            if (i > il || lane != 0) return;
+            if (i > il) return;
             uint64_t* fb = bar + (i & (kAux - 1));
-            unsigned char* d = dsm + (i & (kState - 1)) * Y::state;
-            unsigned char* a = dsm + Y::o_aux + (i & (kAux - 1)) * Y::aux;
-            mbar_arrive_expect_tx(fb, tx);
-            tma_load_3d(d, &M.qx, fb, xs, rf + i, 0);
-            tma_load_3d(d + Y::fs, &M.qy, fb, xs, rf + i, 0);
-            tma_load_3d(d + 2 * Y::fs, &M.p, fb, xs, rf + i, 0);
-            tma_load_3d(d + 3 * Y::fs, &M.u, fb, x4, rf + i, 0);
-            tma_load_3d(a, &M.C, fb, x4, rf + i, 0);
-            tma_load_3d(a + Y::f4, &M.ps, fb, x4, rf + i, 0);
-            if (has_al) tma_load_3d(a + Y::f4 + Y::f1, &M.al, fb, x4, rf + i, 0);
+            if (lane == 0) mbar_arrive_expect_tx(fb, tx);
+            __syncwarp();
+            unsigned char* d =
+                dsm + moff + (lane < 4 ? (i & (kState - 1)) * Y::state : (i & (kAux - 1)) * Y::aux);
+            if (lane < nmaps) tma_load_3d(d, map, fb, mx, rf + i, 0);
         };
         int issued = 0;  // input rows issued
         if (inputs)
