@@ -123,7 +123,9 @@ typedef struct {
                           iterations per launch; Potts with at most 16 labels
                           and float32 cost planes (odd widths: rpADMMII,
                           rpADMMI, pADMMI): labels side by side, two iterations
-                          per launch; both with the results of the variant that
+                          per launch; rPDRQ of one sweep at even widths (Potts:
+                          the same label and cost limits): rows brought ahead
+                          by TMA; all with the results of the variant that
                           would follow: warp strips where the layout allows
                           them (binary ADMM: two iterations per launch), else
                           TMA-staged tiles (Potts, and binary grids
@@ -201,10 +203,12 @@ typedef struct {
                           also with phase_gap = 1.5 tol_gap (the switch left
                           to the first phase's stall test).  Other algorithms
                           ignore it.                                         */
-    int batch_rows;    /* cmf_solve_batch: band height of the warp-strip items
-                          of its Potts instances, 8..24 (0 = 24); the items
-                          of a band share its halo rows, the warps of a batch
-                          share the work of small instances.               */
+    int batch_rows;    /* cmf_solve_batch: band height of the items of its
+                          Potts ADMM instances, 8..24; 0 or 24: warp strips 24,
+                          labels side by side as many rows as the instances
+                          still active call for.  The items of a band share its
+                          halo rows, the warps of a batch share the work of
+                          small instances.                                  */
 } cmf_params;
 
 /* Fill *p with the paper's defaults for `algo` and L labels (L = 2 for the
@@ -424,7 +428,9 @@ typedef struct {
 
 /* Workspace bytes for a batch (0 when an instance or the parameters are
  * invalid).  The batch runs the fused kernels (p->impl = CMF_FUSED), needs an
- * even p->check_every that divides p->max_iter, and for rPDRQ one sweep. */
+ * even p->check_every that divides p->max_iter, and for rPDRQ one sweep.
+ * The size holds the tensor maps of the instances; a smaller workspace that
+ * still holds everything else solves with the kernels that need none. */
 size_t cmf_batch_workspace_bytes(const cmf_instance *inst, int n, const cmf_params *p);
 
 /* Solve all n instances (host array; device pointers inside) with the same
@@ -434,7 +440,8 @@ size_t cmf_batch_workspace_bytes(const cmf_instance *inst, int n, const cmf_para
  * the step bound cmf_default_params takes for their L);
  * cold start unless p->warm_start.  Fills the
  * result fields of every instance.  Returns CMF_OK when every instance
- * reached p->tol_gap, CMF_NOT_CONVERGED when some stopped at max_iter. */
+ * reached p->tol_gap, CMF_NOT_CONVERGED when some stopped at max_iter,
+ * CMF_ETIMEOUT when a bounded device-side wait ran out. */
 cmf_status cmf_solve_batch(cmf_instance *inst, int n, const cmf_params *p, void *d_ws,
                            size_t ws_bytes, void *stream);
 

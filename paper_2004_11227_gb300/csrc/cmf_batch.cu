@@ -2,10 +2,13 @@
 // count advanced together inside one CUDA graph (conditional WHILE node), with
 // per-instance convergence masks.
 //
-// Every iteration launches one kernel over the tiles of all binary instances,
-// one over the tiles of the Potts instances that run on tiles (odd widths,
-// rPDRQ) and one over the warp-strip items of the other Potts instances; a
-// block (tiles) or warp (strip items) maps its work to an instance through a
+// Instances whose layout allows it run the kernels of the single solves (chains
+// of warps; labels side by side, in classes of at most 4, 8 and 16 labels), each
+// kind on a branch of the graph of its own, since no kind waits for another.  The
+// rest (rPDRQ, more than 16 labels, layouts those kernels refuse, a workspace
+// without room for the tensor maps) run one kernel over the tiles of the binary
+// instances, one over the tiles of the Potts instances and one over their
+// warp-strip items; a block or warp maps its work to an instance through a
 // device table and skips it when that instance has converged.  Every
 // check_every iterations the strip instances' multipliers are turned back from
 // the w form into u, the certificates of all instances are computed tile by
@@ -15,7 +18,6 @@
 #include <string.h>
 
 #include <functional>
-#include <initializer_list>
 #include <vector>
 
 #include "cmf_kernels.cuh"
@@ -35,7 +37,8 @@ struct BatchLayout {
     bool chains;
     int n_maps, n_chain_items, chain_rows;
     int n_rows_items;  // room for their items (at bands of at most 12 rows)
-    int rows_rows[3], rows_labels[3];
+    int rows_rows, rows_labels[3];
+    bool rows_fixed;  // params.batch_rows asks for these bands
 };
 
 // Whether a Potts instance of a batch runs by warp strips (the ADMM family,
@@ -81,18 +84,30 @@ bool batch_chain(const cmf_instance& in, const cmf_params& p) {
     return binary_chain_eligible(P, p.storage, s, s, s);
 }
 constexpr int kSideCols = 56;  // columns a strip of the labels side by side advances
-// Band height for instances of a class that together have `rows` strip rows:
-// rounds of the blocks a GB300 holds, each costing the band and the rows that
-// fill and drain it; ties to lower bands (they spread a batch's last, small
-// instances wider).
-int band_rows(long long rows, long long resident, int fill, std::initializer_list<int> heights) {
-    int best = 0;
+// Base bands of the instances on the single solves' kernels: three classes of
+// label counts, chains.  A block takes `merge` base bands of its strip, as many as
+// the instances still active call for (k_batch_decide); the blocks of the others
+// leave at once.  A batch's bulk wants tall bands (a block's nine rows of fill
+// weigh less), its tail short ones (more blocks); one height for a whole batch,
+// 12 to 48 rows, took 263 / 577 / 2682 ms for 16 / 64 / 256 uneven instances,
+// this 203 / 462 / 2078.
+constexpr int kBaseRows = 12, kChainRows = 16, kMostBands = 8192;
+struct MergeRule {
+    int rows[4];  // base band heights; 0: one band a block (params.batch_rows)
+};
+// Base bands of `base` rows a block should take when the active instances have
+// `rows` strip rows in all: rounds of the blocks a GB300 holds, each costing the
+// band and the rows that fill and drain it; ties to shorter bands.
+__device__ int merge_for(long long rows, int base, int resident, int fill) {
+    const int f[9] = {1, 2, 3, 4, 6, 8, 12, 16, 22};
+    int best = 1;
     long long cost = -1;
-    for (int r : heights) {
+    for (int k = 0; k < 9; ++k) {
+        const int r = base * f[k];
         const long long c = ((rows + r - 1) / r + resident - 1) / resident * (r + fill);
         if (cost < 0 || c < cost) {
             cost = c;
-            best = r;
+            best = f[k];
         }
     }
     return best;
@@ -113,22 +128,23 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
                          bool chains = true) {
     BatchLayout b{};
     b.chains = chains;
-    long long side_rows[3] = {0, 0, 0}, chain_rows = 0;
+    long long strip_rows_all = 0;
     for (int i = 0; chains && i < n; ++i) {
         const cmf_instance& in = inst[i];
         const int k = rows_class(in.L);
-        if (batch_side(in, p)) {
-            side_rows[k] += (long long)((in.W + kSideCols - 1) / kSideCols) * in.H;
-            if (in.L > b.rows_labels[k]) b.rows_labels[k] = in.L;
-        } else if (batch_chain(in, p)) {
-            chain_rows += (long long)((in.W + batch_chain_cols() - 1) / batch_chain_cols()) * in.H;
-        }
+        if (!batch_side(in, p)) continue;
+        strip_rows_all += (long long)((in.W + kSideCols - 1) / kSideCols) * in.H;
+        if (in.L > b.rows_labels[k]) b.rows_labels[k] = in.L;
     }
-    for (int k = 0; k < 3; ++k)
-        b.rows_rows[k] = p.batch_rows > 0 ? p.batch_rows
-                                          : band_rows(side_rows[k], 152 * (3 - k), 8,
-                                                      {12, 16, 24, 32, 48});
-    b.chain_rows = band_rows(chain_rows, 152 * 4, 14, {8, 16, 24, 32, 48, 64});
+    b.rows_fixed = p.batch_rows > 0 && p.batch_rows < potts_strip_max_rows();
+    // base bands are taller where there would be more than kMostBands of them:
+    // the blocks that leave at once cost time too (256 instances of the uneven
+    // workload: 12 rows 2284 ms, this rule 2078)
+    b.rows_rows = kBaseRows;
+    while (b.rows_rows < 4 * kBaseRows && strip_rows_all / b.rows_rows > kMostBands)
+        b.rows_rows *= 2;
+    if (b.rows_fixed) b.rows_rows = p.batch_rows;
+    b.chain_rows = kChainRows;
     int maxL = 2;
     for (int i = 0; i < n; ++i)
         if (inst[i].model == 1 && inst[i].L > maxL) maxL = inst[i].L;
@@ -150,9 +166,9 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
             }
             b.n_bin_ev += ev;
         } else {
-            const int ty = 8 * b.potts_rows, k = rows_class(in.L);
+            const int ty = 8 * b.potts_rows;
             if (chains && batch_side(in, p)) {
-                const int r = b.rows_rows[k] < 12 ? b.rows_rows[k] : 12;
+                const int r = b.rows_rows < kBaseRows ? b.rows_rows : kBaseRows;
                 b.n_rows_items += (in.W + kSideCols - 1) / kSideCols * ((in.H + r - 1) / r);
                 ++b.n_maps;
             } else if (batch_strip(in, p))
@@ -187,9 +203,32 @@ struct BatchCtl {
     int it;
     int stop;
     int err;  // kErrWaitTimeout: a bounded device-side wait ran out
+    int merge[4];  // base bands a block takes (three classes of label counts, chains)
 };
 
-__global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl) {
+// One block: how many base bands a block takes, from the instances still active.
+__device__ void set_merge(const BatchDesc* desc, int n, const MergeRule& rule, BatchCtl* ctl) {
+    __shared__ unsigned long long rows[4];
+    if (threadIdx.x < 4) rows[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const BatchDesc& D = desc[i];
+        if (!D.active || D.maps < 0) continue;
+        const int k = D.model == 0 ? 3 : (D.pp.L <= 4 ? 0 : (D.pp.L <= 8 ? 1 : 2));
+        const int H = D.model == 0 ? D.bp.g.H : D.pp.g.H;
+        atomicAdd(&rows[k], (unsigned long long)D.sp_nstrips * (unsigned long long)H);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        const int k = threadIdx.x;
+        ctl->merge[k] = rule.rows[k] == 0
+                            ? 1
+                            : merge_for((long long)rows[k], rule.rows[k],
+                                        k == 3 ? 152 * 4 : 152 * (3 - k), k == 3 ? 14 : 8);
+    }
+}
+
+__global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl, MergeRule rule) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         desc[i].active = 1;
         desc[i].iters = 0;
@@ -199,6 +238,8 @@ __global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl) {
         ctl->it = 0;
         ctl->stop = 0;
     }
+    __syncthreads();
+    set_merge(desc, n, rule, ctl);
 }
 
 // One block per instance: sum its certificate partials in index order.
@@ -238,8 +279,8 @@ __global__ void k_batch_reduce(const BatchDesc* desc, const double* partials, do
 // One block: retire converged instances, decide whether the loop runs again.
 // set_h = 0: a host-driven loop (no graph), which reads ctl->stop instead.
 __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, BatchCtl* ctl, int K,
-                               int max_iter, double tol, cudaGraphConditionalHandle h,
-                               int set_h) {
+                               int max_iter, double tol, MergeRule rule,
+                               cudaGraphConditionalHandle h, int set_h) {
     const int it = ctl->it + K;
     int any = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -263,6 +304,7 @@ __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, Batch
         }
     }
     any = __syncthreads_or(any);
+    set_merge(desc, n, rule, ctl);
     if (threadIdx.x == 0) {
         ctl->it = it;
         ctl->stop = any ? 0 : 1;
@@ -422,7 +464,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
                 const int k = rows_class(in.L);
                 D.sp_out = kSideCols;
                 D.sp_nstrips = (in.W + kSideCols - 1) / kSideCols;
-                D.sp_rows = B.rows_rows[k];
+                D.sp_rows = B.rows_rows;
                 D.maps = (int)maps.size();
                 maps.emplace_back();
                 CMF_CUDA_TRY(potts_rows_maps(D.pp, p->storage, D.pu, maps.back().set[0].potts));
@@ -492,7 +534,10 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
                 CMF_CUDA_TRY(potts_init(p->storage, D.pp, D.pu, dr, (float)p->tau, st));
         }
     }
-    k_batch_reset<<<1, 256, 0, st>>>(d_desc, n, ctl);
+    MergeRule rule;
+    for (int k = 0; k < 3; ++k) rule.rows[k] = B.rows_fixed ? 0 : B.rows_rows;
+    rule.rows[3] = B.chain_rows;
+    k_batch_reset<<<1, 256, 0, st>>>(d_desc, n, ctl, rule);
     CMF_CUDA_TRY(cudaGetLastError());
 
     // coefficients shared by the instances on the single solves' kernels (their
@@ -540,7 +585,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
                     const int it = k < singles ? 1 : 2;
                     e = batch_potts_rows_step(p->storage, aniso, 4 << c, B.rows_labels[c], it,
                                               d_desc, d_maps, d_ritems[c], (int)ritems[c].size(),
-                                              Ks, m & 1, k == 0, &ctl->err, s);
+                                              Ks, m & 1, k == 0, &ctl->merge[c], &ctl->err, s);
                     k += it;
                 }
                 return e;
@@ -554,7 +599,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             for (int m = 0; m < nl && e == cudaSuccess; ++m)
                 e = batch_binary_chain_step(p->storage, aniso, K / nl + (m < K % nl ? 1 : 0),
                                             d_desc, d_maps, d_citems, (int)citems.size(), Ks,
-                                            m & 1, &ctl->err, s);
+                                            m & 1, &ctl->merge[3], &ctl->err, s);
             return e;
         });
     // one chunk: check_every iterations of every active instance, the
@@ -589,7 +634,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         if (e == cudaSuccess) {
             k_batch_reduce<<<n, 256, 0, s>>>(d_desc, partials, scal);
             k_batch_decide<<<1, 256, 0, s>>>(d_desc, n, scal, ctl, p->check_every, p->max_iter,
-                                              p->tol_gap, h, set_h);
+                                              p->tol_gap, rule, h, set_h);
             e = cudaGetLastError();
         }
         return e;

@@ -5,25 +5,25 @@ namespace cmf {
 
 cudaError_t batch_rows_f32(
     bool aniso, int lc, int nlab, int iters, const BatchDesc* desc, const BatchMaps* maps,
-    const int2* items, int nitems, const AdmmCoef& K, int parity, int first, int* err,
-    cudaStream_t st);
+    const int2* items, int nitems, const AdmmCoef& K, int parity, int first,
+    const int* merge, int* err, cudaStream_t st);
 cudaError_t batch_chain_f32(
     bool aniso, int T, const BatchDesc* desc, const BatchMaps* maps, const int2* items, int nitems,
-    const AdmmCoef& K, int parity, int* err, cudaStream_t st);
+    const AdmmCoef& K, int parity, const int* merge, int* err, cudaStream_t st);
 cudaError_t batch_rows_f16(
     bool aniso, int lc, int nlab, int iters, const BatchDesc* desc, const BatchMaps* maps,
-    const int2* items, int nitems, const AdmmCoef& K, int parity, int first, int* err,
-    cudaStream_t st);
+    const int2* items, int nitems, const AdmmCoef& K, int parity, int first,
+    const int* merge, int* err, cudaStream_t st);
 cudaError_t batch_chain_f16(
     bool aniso, int T, const BatchDesc* desc, const BatchMaps* maps, const int2* items, int nitems,
-    const AdmmCoef& K, int parity, int* err, cudaStream_t st);
+    const AdmmCoef& K, int parity, const int* merge, int* err, cudaStream_t st);
 cudaError_t batch_rows_bf16(
     bool aniso, int lc, int nlab, int iters, const BatchDesc* desc, const BatchMaps* maps,
-    const int2* items, int nitems, const AdmmCoef& K, int parity, int first, int* err,
-    cudaStream_t st);
+    const int2* items, int nitems, const AdmmCoef& K, int parity, int first,
+    const int* merge, int* err, cudaStream_t st);
 cudaError_t batch_chain_bf16(
     bool aniso, int T, const BatchDesc* desc, const BatchMaps* maps, const int2* items, int nitems,
-    const AdmmCoef& K, int parity, int* err, cudaStream_t st);
+    const AdmmCoef& K, int parity, const int* merge, int* err, cudaStream_t st);
 
 int batch_chain_cols() {
     return chain::kCols - chain::left_cols(chain::kMaxIters) -
@@ -32,21 +32,22 @@ int batch_chain_cols() {
 
 cudaError_t batch_potts_rows_step(int storage, bool aniso, int lc, int nlab, int iters,
                                   const BatchDesc* desc, const BatchMaps* maps, const int2* items,
-                                  int nitems, const AdmmCoef& K, int parity, int first, int* err,
-                                  cudaStream_t st) {
+                                  int nitems, const AdmmCoef& K, int parity, int first,
+                                  const int* merge, int* err, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     auto f = storage == CMF_F32 ? batch_rows_f32
                                 : (storage == CMF_F16 ? batch_rows_f16 : batch_rows_bf16);
-    return f(aniso, lc, nlab, iters, desc, maps, items, nitems, K, parity, first, err, st);
+    return f(aniso, lc, nlab, iters, desc, maps, items, nitems, K, parity, first, merge, err, st);
 }
 
 cudaError_t batch_binary_chain_step(int storage, bool aniso, int T, const BatchDesc* desc,
                                     const BatchMaps* maps, const int2* items, int nitems,
-                                    const AdmmCoef& K, int parity, int* err, cudaStream_t st) {
+                                    const AdmmCoef& K, int parity, const int* merge,
+                                    int* err, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     auto f = storage == CMF_F32 ? batch_chain_f32
                                 : (storage == CMF_F16 ? batch_chain_f16 : batch_chain_bf16);
-    return f(aniso, T, desc, maps, items, nitems, K, parity, err, st);
+    return f(aniso, T, desc, maps, items, nitems, K, parity, merge, err, st);
 }
 
 }  // namespace cmf

@@ -5,16 +5,17 @@ namespace cmf {
 
 cudaError_t batch_rows_f32(
     bool aniso, int lc, int nlab, int iters, const BatchDesc* desc, const BatchMaps* maps,
-    const int2* items, int nitems, const AdmmCoef& K, int parity, int first, int* err,
-    cudaStream_t st) {
+    const int2* items, int nitems, const AdmmCoef& K, int parity, int first,
+    const int* merge, int* err, cudaStream_t st) {
     return batch_rows_s<float>(aniso, lc, nlab, iters, desc, maps, items, nitems, K, parity, first,
-                             err, st);
+                             merge, err, st);
 }
 
 cudaError_t batch_chain_f32(
     bool aniso, int T, const BatchDesc* desc, const BatchMaps* maps, const int2* items, int nitems,
-    const AdmmCoef& K, int parity, int* err, cudaStream_t st) {
-    return batch_chain_s<float>(aniso, T, desc, maps, items, nitems, K, parity, err, st);
+    const AdmmCoef& K, int parity, const int* merge, int* err,
+    cudaStream_t st) {
+    return batch_chain_s<float>(aniso, T, desc, maps, items, nitems, K, parity, merge, err, st);
 }
 
 }  // namespace cmf

@@ -1,5 +1,8 @@
 // Binary ADMM iteration by warp strips (Eq. rpADMMII, Eq. rpADMMI, pADMM-TY
-// Eq. ADMM:Tai_yuan).
+// Eq. ADMM:Tai_yuan): variant 2, and the single iterations of calls that run
+// cmf_binary_strip2.cu.  The rPDRQ strips below run variant 2, two to four
+// sweeps, and rows or planes that are not 16-byte aligned (otherwise
+// cmf_binary_dr_rows.cu).
 //
 // Work unit: one warp, a strip of 64 columns (two adjacent columns per lane)
 // and a band of R output rows, streamed top-down.  Step t holds rows t and

@@ -556,13 +556,14 @@ int potts_strip_max_rows();  // band rows the strip kernels take at most
 // nlab: the most labels among them, K: the coefficients but for a_2.
 cudaError_t batch_potts_rows_step(int storage, bool aniso, int lc, int nlab, int iters,
                                   const BatchDesc* desc, const BatchMaps* maps, const int2* items,
-                                  int nitems, const AdmmCoef& K, int parity, int first, int* err,
-                                  cudaStream_t st);
+                                  int nitems, const AdmmCoef& K, int parity, int first,
+                                  const int* merge, int* err, cudaStream_t st);
 // Binary instances by chains of warps: T iterations (strips of
 // batch_chain_cols() columns).
 cudaError_t batch_binary_chain_step(int storage, bool aniso, int T, const BatchDesc* desc,
                                     const BatchMaps* maps, const int2* items, int nitems,
-                                    const AdmmCoef& K, int parity, int* err, cudaStream_t st);
+                                    const AdmmCoef& K, int parity, const int* merge, int* err,
+                                    cudaStream_t st);
 int batch_chain_cols();
 
 cudaError_t batch_binary_eval(int storage, bool aniso, bool dr, float tau,

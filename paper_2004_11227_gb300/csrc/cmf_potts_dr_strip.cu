@@ -1,7 +1,9 @@
 // Potts rPDRQ iteration by warp strips (Eq. pdrq:4labels, general L): the
 // pipelined red-black Gauss-Seidel preconditioner of Sec. 3 streamed down a
 // band of rows, with the labels of one band shared out among the warps of a
-// block.
+// block.  Runs variant 2, two to four sweeps, more than 16 labels, costs made
+// from the image, and rows or planes that are not 16-byte aligned (otherwise
+// cmf_potts_dr_rows.cuh).
 //
 // Work unit: one block, a strip of 64 columns (two adjacent columns per lane;
 // SW+1 halo lanes on each side) and a band of R output rows.  Phase 1: U =
