@@ -305,38 +305,49 @@ __global__ void __launch_bounds__(kStripWarps * 32, 3)
 }
 
 // u_i = w_i + cu p_s on the owned pixels of every item of an active strip
-// instance (the state is in the caller's buffers after an even chunk).
-__global__ void k_batch_potts_strip_finalize(const BatchDesc* __restrict__ desc,
-                                             const int2* __restrict__ items, int nitems) {
+// instance (the state is in the caller's buffers after an even chunk).  Bound by
+// latency when few instances are left: a block takes an item, its warps the rows
+// in turn, four labels' loads in flight (a warp an item, label by label: 56 us
+// for twelve instances of 4.4 M label-pixels, 13 us so).
+constexpr int kFinWarps = 8;
+__global__ void __launch_bounds__(32 * kFinWarps)
+    k_batch_potts_strip_finalize(const BatchDesc* __restrict__ desc,
+                                 const int2* __restrict__ items) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    for (int it = blockIdx.x * kStripWarps + wib; it < nitems; it += gridDim.x * kStripWarps) {
-        const int2 e = items[it];
-        const BatchDesc* D = desc + e.x;
-        if (!D->active) continue;
-        const Grid G = D->pp.g;
-        const int r0 = (e.y / D->sp_nstrips) * D->sp_rows;
-        const int r1 = min(r0 + D->sp_rows, G.H);
-        const int c = (e.y % D->sp_nstrips) * D->sp_out + 2 * lane;
-        if (2 * lane >= D->sp_out || c >= G.W) continue;
-        const float cu = D->ak.cu;
-        float* u = D->pu.u;
-        const float* ps = D->pu.ps;
-        const bool pair = c + 1 < G.W;  // else the last column of an odd width alone
-        for (int r = r0; r < r1; ++r) {
-            const size_t k = G.idx(r, c);
-            if (pair) {
-                const float2 s = Pair<float>::ld(ps + k);
-                for (int l = 0; l < D->pp.L; ++l) {
-                    float2* q = reinterpret_cast<float2*>(u + (size_t)l * G.plane + k);
-                    float2 v = *q;
-                    v.x += cu * s.x;
-                    v.y += cu * s.y;
-                    *q = v;
+    const int2 e = items[blockIdx.x];
+    const BatchDesc* D = desc + e.x;
+    if (!D->active) return;
+    const Grid G = D->pp.g;
+    const int L = D->pp.L;
+    const int r0 = (e.y / D->sp_nstrips) * D->sp_rows;
+    const int r1 = min(r0 + D->sp_rows, G.H);
+    const int c = (e.y % D->sp_nstrips) * D->sp_out + 2 * lane;
+    if (2 * lane >= D->sp_out || c >= G.W) return;
+    const float cu = D->ak.cu;
+    float* const u = D->pu.u;
+    const float* const ps = D->pu.ps;
+    const bool pair = c + 1 < G.W;  // else the last column of an odd width alone
+    for (int r = r0 + wib; r < r1; r += kFinWarps) {
+        const size_t k = G.idx(r, c);
+        if (pair) {
+            const float2 s = Pair<float>::ld(ps + k);
+            for (int l = 0; l < L; l += 4) {
+                float2 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (l + i < L)
+                        v[i] = *reinterpret_cast<const float2*>(u + (size_t)(l + i) * G.plane + k);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (l + i >= L) break;
+                    v[i].x += cu * s.x;
+                    v[i].y += cu * s.y;
+                    *reinterpret_cast<float2*>(u + (size_t)(l + i) * G.plane + k) = v[i];
                 }
-            } else {
-                const float s = ps[k];
-                for (int l = 0; l < D->pp.L; ++l) u[(size_t)l * G.plane + k] += cu * s;
             }
+        } else {
+            const float s = ps[k];
+            for (int l = 0; l < L; ++l) u[(size_t)l * G.plane + k] += cu * s;
         }
     }
 }
@@ -393,14 +404,7 @@ cudaError_t batch_potts_strip_step(int storage, bool aniso, bool odd_width, cons
 cudaError_t batch_potts_strip_finalize(const BatchDesc* desc, const int2* items, int nitems,
                                        cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
-    int dev = 0, sms = 0;
-    cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return e;
-    const int blocks = (nitems + kStripWarps - 1) / kStripWarps;
-    const int grid = blocks < 8 * sms ? blocks : 8 * sms;
-    k_batch_potts_strip_finalize<<<grid, kStripWarps * 32, 0, st>>>(desc, items, nitems);
+    k_batch_potts_strip_finalize<<<nitems, 32 * kFinWarps, 0, st>>>(desc, items);
     return cudaGetLastError();
 }
 
