@@ -322,7 +322,7 @@ KERNEL_CASES = {
 def binary_workload(cmf, synth, flush, peak) -> dict:
     """The binary 1024^2 workload (eight disks / rectangles, edge-weighted
     alpha): time to the 1e-4 gap of every algorithm, fused and plain, and the
-    two-iterations-per-launch warp-strip kernel's bandwidth.  Its state (about
+    chain kernel's bandwidth (four iterations per launch).  Its state (about
     75 MB) stays in the 129 MB L2, so the bound is L2, not HBM."""
     import torch
 
@@ -346,22 +346,22 @@ def binary_workload(cmf, synth, flush, peak) -> dict:
     t = out["time_to_gap_ms"]
     out["speedup_fused_vs_plain_rpADMMII"] = round(t["rpADMMII_plain"]["ms"] /
                                                    t["rpADMMII_fused"]["ms"], 3)
-    # the fused kernel: 200 iterations = 100 two-iteration launches, back to back
+    # the fused kernel: 200 iterations = 50 four-iteration launches, back to back
     p = cmf.default_params(FLAGSHIP, 2)
     b = cmf.alloc_binary(inst, p)
     cmf.cmf_init_binary(b)
     cmf.cmf_iterate_binary(b, 20)
     flush.zero_()
     ms, _ = _timed(lambda: cmf.cmf_iterate_binary(b, 200))
-    launch_ms = ms / 100
-    nbytes = 2 * algorithmic_bytes_per_px("binary", 2, 0, True) * inst.H * inst.W
-    out["roofline"] = {"bound": "l2", "kernel": "k_binary_strip2", "launch_ms": launch_ms,
-                       "iterations_per_launch": 2, "algorithmic_bytes_per_launch": nbytes,
+    launch_ms = ms / 50
+    nbytes = 4 * algorithmic_bytes_per_px("binary", 2, 0, True) * inst.H * inst.W
+    out["roofline"] = {"bound": "l2", "kernel": "k_binary_chain", "launch_ms": launch_ms,
+                       "iterations_per_launch": 4, "algorithmic_bytes_per_launch": nbytes,
                        "achieved": nbytes / launch_ms / 1e6, "unit": "GB/s",
                        "frac_of_hbm_peak": nbytes / launch_ms / 1e6 / peak,
-                       "traffic": _traffic("paper_2004_11227_gb300/csrc/cmf_binary_strip2.cu",
-                                           "k_binary_strip2"),
-                       "note": "effective: iteration k+1 stays on chip and the state in L2"}
+                       "traffic": _traffic("paper_2004_11227_gb300/csrc/cmf_binary_chain.cuh",
+                                           "k_binary_chain"),
+                       "note": "effective: three of four iterations stay on chip, the state in L2"}
     return out
 
 
@@ -369,7 +369,7 @@ def potts4_workload(cmf, synth, flush, peak) -> dict:
     """The 4-label 2048^2 Voronoi workload (alpha 0.3): per flow storage the
     fused iteration's time and bandwidth and the time to the 1e-4 gap, the
     plain float32 form's time to the gap, and the same for rPDRQ (one
-    red-black sweep, fused: k_potts_dr_strip)."""
+    red-black sweep, fused: k_potts_dr_rows)."""
     inst = synth.config3()
     out = {"workload": "potts L=4 2048x2048 Voronoi (64 seeds), alpha 0.3, solve to gap 1e-4"}
     for algo, storage, name, impl, max_iter in ((FLAGSHIP, 0, "float32", 0, 20000),
@@ -842,10 +842,10 @@ def main():
     iters = int(np.median(iters_all))
     it16 = int(np.median(phase1))
     # per solve: cold start, two loop resets, the float16-to-float32 switch;
-    # per check: check_every iteration launches, the launch that turns w back
-    # into u, the certificate launch (its last block reduces and takes the
-    # stop decision)
-    launches = args.steps * (4 + (iters // CHECK_EVERY) * (CHECK_EVERY + 2))
+    # per check: 24 launches of two iterations and two of one (an even number ends
+    # in the caller's buffers), the launch that turns w back into u, the
+    # certificate launch (its last block reduces and takes the stop decision)
+    launches = args.steps * (4 + (iters // CHECK_EVERY) * (CHECK_EVERY // 2 + 3))
 
     # --- end to end through the C ABI with host buffers -------------------------------
     cdt = s.C.dtype
@@ -890,7 +890,8 @@ def main():
     ms16, ms32 = kernel_ms(1), kernel_ms(0)
     t16, t32 = ms16 * it16, ms32 * (iters - it16)
     storage_dom = 1 if t16 >= t32 else 0
-    launch_ms = ms16 if storage_dom == 1 else ms32
+    # a launch makes two iterations and moves the state once for both
+    launch_ms = 2 * (ms16 if storage_dom == 1 else ms32)
     # algorithmic bytes of the dominant instantiation: for float32 every field
     # in 4 bytes (u, q_i, p_i, p_s read and written, costs and alpha read:
     # 16 x 36 + 8 + 4 = 588 B/px); for the float16 phase q_i and p_i in 2 bytes
@@ -901,28 +902,30 @@ def main():
     design_px = algorithmic_bytes_per_px("potts", L, storage_dom, True,
                                          {0: "f32", 2: "f16"}[COSTS])
     achieved = algo_px * H * W / (launch_ms / 1000.0) / 1e9
-    name = "k_potts_strip<__half>" if storage_dom == 1 else "k_potts_strip<float>"
+    name = "k_potts_rows<__half>" if storage_dom == 1 else "k_potts_rows<float>"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak,
-                "traffic": _traffic("paper_2004_11227_gb300/csrc/cmf_potts_strip.cu", name),
+                "traffic": _traffic("paper_2004_11227_gb300/csrc/cmf_potts_rows.cuh", name),
                 "kernel": name, "peak_kind": peak_kind,
                 "algorithmic_bytes_per_px": algo_px,
                 "algorithmic_bytes_per_launch": algo_px * H * W, "launch_ms": launch_ms,
+                "iterations_per_launch": 2,
                 "design_bytes_per_px": design_px,
                 "time_share_in_solve": {"float16_phase": t16 / (t16 + t32),
                                         "float32_phase": t32 / (t16 + t32)},
-                "float16_kernel": {"launch_ms": ms16, "bytes_per_px_16bit": BYTES_PER_PX_16BIT,
-                                   "frac_16bit_count": BYTES_PER_PX_16BIT * H * W / ms16 / 1e6 / peak,
+                "float16_kernel": {"launch_ms": 2 * ms16, "bytes_per_px_16bit": BYTES_PER_PX_16BIT,
+                                   "frac_16bit_count": BYTES_PER_PX_16BIT * H * W / ms16 / 2e6 / peak,
                                    "design_bytes_per_px": algorithmic_bytes_per_px(
                                        "potts", L, 1, True, {0: "f32", 2: "f16"}[COSTS]),
                                    "frac_design": algorithmic_bytes_per_px(
                                        "potts", L, 1, True, {0: "f32", 2: "f16"}[COSTS]) *
-                                   H * W / ms16 / 1e6 / peak},
-                "float32_kernel": {"launch_ms": ms32,
+                                   H * W / ms16 / 2e6 / peak},
+                "float32_kernel": {"launch_ms": 2 * ms32,
                                    "frac": algorithmic_bytes_per_px("potts", L, 0, True, "f32") *
-                                   H * W / ms32 / 1e6 / peak},
-                "note": "launch time = 50 back-to-back iterations / 50 (one w-to-u pass per "
-                        "call included); the dominant instantiation by time in the solve"}
+                                   H * W / ms32 / 2e6 / peak},
+                "note": "launch time = 50 back-to-back iterations / 25 (one w-to-u pass per "
+                        "call included); a launch makes two iterations, its bytes are those "
+                        "of one; the dominant instantiation by time in the solve"}
 
     side = {}
     if rank == 0 and not args.skip_side:
