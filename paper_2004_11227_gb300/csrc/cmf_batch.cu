@@ -213,7 +213,7 @@ __device__ void set_merge(const BatchDesc* desc, int n, const MergeRule& rule, B
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const BatchDesc& D = desc[i];
-        if (!D.active || D.maps < 0) continue;
+        if (!D.active || !D.sp_maps) continue;
         const int k = D.model == 0 ? 3 : (D.pp.L <= 4 ? 0 : (D.pp.L <= 8 ? 1 : 2));
         const int H = D.model == 0 ? D.bp.g.H : D.pp.g.H;
         atomicAdd(&rows[k], (unsigned long long)D.sp_nstrips * (unsigned long long)H);
@@ -435,7 +435,8 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
                 D.sp_out = batch_chain_cols();
                 D.sp_nstrips = (in.W + D.sp_out - 1) / D.sp_out;
                 D.sp_rows = B.chain_rows;
-                D.maps = (int)maps.size();
+                D.sp_maps = 1;
+                D.tile_base = (int)maps.size();
                 maps.emplace_back();
                 CMF_CUDA_TRY(binary_chain_maps(D.bp, p->storage, D.bu, maps.back().set[0].binary));
                 CMF_CUDA_TRY(binary_chain_maps(D.bp, p->storage, D.bw, maps.back().set[1].binary));
@@ -465,7 +466,8 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
                 D.sp_out = kSideCols;
                 D.sp_nstrips = (in.W + kSideCols - 1) / kSideCols;
                 D.sp_rows = B.rows_rows;
-                D.maps = (int)maps.size();
+                D.sp_maps = 1;
+                D.tile_base = (int)maps.size();
                 maps.emplace_back();
                 CMF_CUDA_TRY(potts_rows_maps(D.pp, p->storage, D.pu, maps.back().set[0].potts));
                 CMF_CUDA_TRY(potts_rows_maps(D.pp, p->storage, D.pw, maps.back().set[1].potts));

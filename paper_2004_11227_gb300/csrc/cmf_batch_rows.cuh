@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(32 * (LC + rows::service_warps(T, LC)),
     const BatchDesc* D = desc + e.x;
     const int band = e.y / D->sp_nstrips, take = *merge;
     if (!D->active || band % take != 0) return;
-    const PottsRowsMaps* M = &maps[D->maps].set[parity].potts;
+    const PottsRowsMaps* M = &maps[D->tile_base].set[parity].potts;
     acquire_maps(&M->qx, sizeof(PottsRowsMaps) / sizeof(CUtensorMap));
     K.inv_a2 = D->ak.inv_a2;
     const PottsProblem P = D->pp;
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(32 * (chain::kMaxIters + 1), 4)
     const BatchDesc* D = desc + e.x;
     const int band = e.y / D->sp_nstrips, take = *merge;
     if (!D->active || band % take != 0) return;
-    const BinChainMaps* M = &maps[D->maps].set[parity].binary;
+    const BinChainMaps* M = &maps[D->tile_base].set[parity].binary;
     acquire_maps(&M->qx, sizeof(BinChainMaps) / sizeof(CUtensorMap));
     const BinProblem P = D->bp;
     const BinState<S> s1 = (parity ? D->bu : D->bw).as<S>();

@@ -508,6 +508,7 @@ struct BatchDesc {
     int active;      // 1 while the instance still iterates
     int ntx;         // 32-wide tile columns
     int tile_base;   // first entry of this instance in its model's iteration tile table
+                     // (sp_maps: index of its tensor map sets)
     int ev_tab;      // first entry in its model's certificate tile table
     int ev_base;     // first certificate partial of this instance
     int ev_count;    // certificate tiles of this instance
@@ -520,9 +521,9 @@ struct BatchDesc {
     AdmmCoef ak;           // coefficients for this instance's L
     DrCoef dk;
     int sp_nstrips;        // Potts by warp strips: strips of the grid (0: tiles)
-    int sp_rows;           // band height of its strip items
-    int sp_out;            // columns a strip advances
-    int maps;              // index of its tensor map sets (chains, labels side by side), or -1
+    unsigned short sp_rows;  // band height of its strip items
+    unsigned char sp_out;    // columns a strip advances
+    unsigned char sp_maps;   // 1: chains, labels side by side (they use tensor maps)
 };
 
 // Tensor maps of a batch instance: the caller's state and the workspace's.
