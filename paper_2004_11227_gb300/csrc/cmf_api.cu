@@ -212,7 +212,7 @@ struct BinaryCall {
     bool strip;             // fused ADMM by warp strips
     bool pairs;             // warp strips, two ADMM iterations per launch
     bool chain;             // chains of warps, up to four ADMM iterations per launch
-    bool dr_rows;           // rPDRQ on warp-private TMA rings
+    bool dr_rows;           // rPDRQ on shared TMA rows
     BinChainMaps cmaps[3];  // tensor maps of the buffer sets
     int cert_blocks;        // partial triples the workspace holds
     BinTmaMaps maps[2];     // tensor maps of the user / workspace state sets
@@ -543,11 +543,13 @@ struct PottsCall {
 };
 
 // `layout`: the parameters the workspace was sized for (default *p); `set`:
-// the second state set (default: the workspace's own, in p->storage).
+// the second state set (default: the workspace's own, in p->storage); `certs`:
+// whether certificates may follow.
 cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0, int H, int W,
                          int pitch, const cmf_params* p, float* u, void* qx, void* qy, void* pp,
                          void* ps, void* ws, size_t ws_bytes, PottsCall& call,
-                         const cmf_params* layout = nullptr, const PottsStateV* set = nullptr) {
+                         const cmf_params* layout = nullptr, const PottsStateV* set = nullptr,
+                         bool certs = true) {
     cmf_status s;
     if (L < 2 || L > 64) return CMF_EINVAL;
     if ((s = check_params(p, L)) != CMF_OK) return s;
@@ -579,16 +581,22 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     // at 4096^2, L = 16, faster at every size measured from 128^2 and L = 2 on,
     // with the same results), else warp strips where the layout allows them,
     // else TMA tiles, else shared-memory tiles
-    call.cert = potts_rows_layout(call.P, p->storage, call.user, call.ws) &&
+    const bool free_choice = !call.cfg.plain && p->variant == 0;
+    const bool dr_rows =
+        free_choice && call.cfg.dr && potts_dr_rows_takes(call.P, call.cfg.dc);
+    const bool rows =
+        free_choice && !call.cfg.dr &&
+        potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws);
+    // the maps: fourteen driver calls, about 4 us, only where a launch reads them
+    call.cert = (certs || rows || dr_rows) &&
+                potts_rows_layout(call.P, p->storage, call.user, call.ws) &&
                 potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
                 potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess;
-    if (!call.cfg.plain && call.cfg.dr && p->variant == 0 && call.cert &&
-        potts_dr_rows_takes(call.P, call.cfg.dc)) {
+    if (dr_rows && call.cert) {
         call.dr_rows = true;
         return CMF_OK;
     }
-    if (!call.cfg.plain && !call.cfg.dr && p->variant == 0 && call.cert &&
-        potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws)) {
+    if (rows && call.cert) {
         call.rows = true;
         call.rfused = potts_rows_fused(call.P, p->storage, call.cfg.aniso);
         return CMF_OK;
@@ -1292,7 +1300,7 @@ cmf_status cmf_iterate_potts(const float* d_C, int L, const float* d_alpha, floa
                              size_t ws_bytes, void* stream) {
     PottsCall c;
     cmf_status s = potts_prepare(d_C, L, d_alpha, alpha0, H, W, pitch, p, d_u, d_qx, d_qy, d_p,
-                                 d_ps, d_ws, ws_bytes, c);
+                                 d_ps, d_ws, ws_bytes, c, nullptr, nullptr, false);
     if (s != CMF_OK) return s;
     if (n_iter < 0) return CMF_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;

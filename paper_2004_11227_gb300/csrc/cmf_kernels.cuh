@@ -397,7 +397,7 @@ cudaError_t binary_chain_step(
 cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s, int cs, int c4,
                             BinChainMaps& m);
 
-// --- binary rPDRQ on warp-private TMA rings (cmf_binary_dr_rows.cu) ---
+// --- binary rPDRQ on shared TMA rows (cmf_binary_dr_rows.cu) ---
 // One iteration from the state of src_maps into b; a bounded wait that runs out
 // sets *err.
 bool binary_dr_rows_eligible(const BinProblem& P, int storage, const DrCoef& D,
