@@ -22,6 +22,8 @@
 //   - a share slot is rewritten four rows on, after its writer has waited for
 //     a p_s that the service warp gave after summing it (T == 2), or for an
 //     input row issued after that (T == 1);
+//   - a service warp that only brings rows waits for the labels' steps no longer
+//     than it has rows to issue (cmf_rows_order.cuh);
 //   - stage B's shares of row s-3 are complete when every label has arrived
 //     for row s.
 // The multipliers travel as w = u - cu p_s between launches, as in the
@@ -48,6 +50,7 @@
 #include <type_traits>
 
 #include "cmf_kernels.cuh"
+#include "cmf_rows_order.cuh"
 #include "cmf_strip.cuh"
 #include "cmf_tma.cuh"
 
@@ -57,10 +60,6 @@ namespace rows {
 using strip::Pair;
 
 constexpr int kMaxLabels = 16;
-constexpr int kState = 4;          // state rows in shared memory
-constexpr int kAux = 8;            // cost / p_s / alpha rows in shared memory
-constexpr int kSh = 4;             // share slots of each stage
-constexpr int kPs = 8;             // p_s^{k+1} rows
 
 // Columns of a staged row segment: 64 plus what aligning its start to 16
 // bytes can put in front.
@@ -90,10 +89,6 @@ struct Layout {
     static constexpr int o_bar = o_ps + kPs * 256;
     static constexpr int bytes = o_bar + 8 * (kAux + 4 + 4) + 128;  // + alignment of the base
 };
-
-// Service warps of a block: two iterations per launch and many labels keep
-// one warp busy with the label sums alone.
-__host__ __device__ constexpr int service_warps(int T, int LC) { return T == 2 && LC > 4 ? 2 : 1; }
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
@@ -295,6 +290,7 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
         };
         float2* const psr = reinterpret_cast<float2*>(dsm + Y::o_ps) + lane;
         for (int k = 0; k <= ke; ++k) {
+            if (!sums && !inputs_wait(issued, il)) break;
             const int s = js + k;
             ok = mbar_wait(b_sf + 8 * (k & 3), (k >> 2) & 1);
             if (!ok) break;
@@ -318,13 +314,13 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
             }
             if (inputs) {
                 __syncwarp();
-                for (; issued <= k + 2 + kState; ++issued) issue(issued);
+                for (; issued < issued_after(k); ++issued) issue(issued);
             }
         }
-        if (!ok && inputs && lane == 0) {
-            // a label never arrived: report it and let the copies in flight
-            // land before the block's shared memory goes
-            atomicExch(err, kErrWaitTimeout);
+        if (!ok && inputs && lane == 0) atomicExch(err, kErrWaitTimeout);  // a label never arrived
+        if ((!ok || !sums) && inputs && lane == 0) {
+            // the copies in flight land before the block's shared memory goes,
+            // whatever becomes of the labels
             issued = min(issued, il + 1);
             for (int i = max(0, issued - kAux); i < issued; ++i)
                 mbar_wait(b_full + 8 * (i & (kAux - 1)), (i / kAux) & 1);
@@ -472,7 +468,7 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
         constexpr int a1 = ((U + 2) & 7) * Y::aux, a0 = ((U + 1) & 7) * Y::aux,
                       ab = ((U + 6) & 7) * Y::aux;
         Row<S>&y2 = y[(U + 2) & 3], &y3 = y[(U + 1) & 3], &yn = y[U & 3];  // rows j-2, j-3, j
-        if (k + 2 <= il)  // row j + 1 (the ones behind rl are made up and not used)
+        if (label_waits_row(k, il))  // row j + 1 (the ones behind rl are made up and not used)
             if (!mbar_wait(b_full + 8 * ((U + 2) & 7), U < 6 ? par : par ^ 1)) return false;
         if (T == 2 && !mbar_wait(b_pr + 8 * (U & 3), U >> 2)) return false;
         if (T == 2) {

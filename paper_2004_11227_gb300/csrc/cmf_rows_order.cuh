@@ -1,0 +1,40 @@
+// Which input rows are issued when, and who waits for whom, in the kernels that
+// couple warps by mbarriers with the labels side by side (cmf_potts_rows.cuh,
+// cmf_potts_cert.cuh): apart from the arithmetic and free of device code, so that
+// a host test can replay the order of events for any schedule of the warps.
+//
+// A wait on an mbarrier tells phases apart by parity alone: a warp that comes to
+// a wait two phases late finds the parity it does not wait for, and waits out the
+// limit.  So whoever waits for a barrier's phase has to be one whom the next phase
+// but one cannot do without.
+#pragma once
+
+#ifdef __CUDACC__
+#define CMF_ORDER __host__ __device__ constexpr
+#else
+#define CMF_ORDER constexpr
+#endif
+
+namespace cmf {
+namespace rows {
+
+constexpr int kState = 4;  // state rows in shared memory
+constexpr int kAux = 8;    // cost / p_s / alpha rows in shared memory
+constexpr int kSh = 4;     // share slots of each stage
+constexpr int kPs = 8;     // p_s^{k+1} rows
+
+// Service warps of a block: two iterations per launch and many labels keep
+// one warp busy with the label sums alone.
+CMF_ORDER int service_warps(int T, int LC) { return T == 2 && LC > 4 ? 2 : 1; }
+// Input rows issued once every label is done with step k: row k + 2 is in the
+// labels' registers, so its state slot is free for the last of them.
+CMF_ORDER int issued_after(int k) { return k + 3 + kState; }
+// Whether a label waits for an input row (k + 2) at step k; il: the last row.
+CMF_ORDER bool label_waits_row(int k, int il) { return k + 2 <= il; }
+// Whether a service warp without the sums still waits for the labels' steps: not
+// once its rows are issued, for from then on no label waits for it, and one that
+// came late would find those steps' barriers used again.
+CMF_ORDER bool inputs_wait(int issued, int il) { return issued <= il; }
+
+}  // namespace rows
+}  // namespace cmf
