@@ -29,11 +29,13 @@
 // instructions per pixel and iteration (60% of the issue slots); odd widths
 // ran one iteration per launch on tiles.  A chain holds one iteration per
 // warp, so four columns a lane fit 96 registers (one address, predicate and
-// shuffle for four pixels): 84 thread instructions, 65% of the issue slots,
-// and the state passes through DRAM once per four iterations (at 4096^2 that
-// floor is 32 us per iteration).  The rest is the barrier (1.3 stalls per
-// issue) and the dependent chain of a row.  Two columns a lane, one or two
-// rows per barrier, took 103-118 instructions.  Small grids are bound by the
+// shuffle for four pixels; float32 spills 4 to 8 bytes, with the certificates
+// up to 60), and the state passes through DRAM once per four iterations (at
+// 4096^2 that floor is 32 us per iteration).  At 1024^2 that is 111 thread
+// instructions with the bands' halo rows, 59% of the issue slots; the rest is
+// the barrier (2.0 to 2.2 stalls per issue) and the dependent chain of a row.  Two
+// columns a lane, one or two rows per barrier, took 1.2 to 1.4 times the
+// instructions.  Small grids are bound by the
 // chain's fill (three steps per iteration) and the launch.  Measured per
 // iteration (CUDA events, float32; before: two iterations per launch by strips,
 // odd widths tiles): 4096^2 87.2 -> 52.2 us, 2048^2 23.8 -> 15.0 us, 1024^2

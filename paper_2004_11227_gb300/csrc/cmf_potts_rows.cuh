@@ -34,9 +34,11 @@
 // iteration at L = 16, float32: 1.45 ms at 4096^2 at the copy bandwidth; it
 // took 2.29 ms); here alpha and p_s are read once and the state moves once per
 // two iterations (half the bytes: 0.73 ms).  What is left is instruction
-// issue and the latency of a row's chain of shuffles: about 230 instructions
-// per warp and row of both stages, four label warps per scheduler (96
-// registers), 50-60% of the issue slots, DRAM at 60-65%.  Hence scalar
+// issue and the latency of a row's chain of shuffles: 75 thread instructions
+// per label-pixel and iteration (float16 flows 83, for the conversions), four
+// label warps per scheduler (96 registers, 4 to 20 bytes of them spilled at two
+// iterations), 59-61% of the issue slots, DRAM at 69% (float16 43%; 2048^2,
+// L = 16).  Hence scalar
 // arithmetic with the coefficients as constant operands (packed float32
 // instructions spent what they saved on register moves), rings whose
 // positions are constants (the row loop is unrolled by their length, eight),
@@ -289,8 +291,9 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
             else o[0] = n.x;
         };
         float2* const psr = reinterpret_cast<float2*>(dsm + Y::o_ps) + lane;
-        for (int k = 0; k <= ke; ++k) {
-            if (!sums && !inputs_wait(issued, il)) break;
+        const int kl = sums ? ke : last_input_step(il);
+        int k = 0;
+        for (; k <= kl; ++k) {
             const int s = js + k;
             ok = mbar_wait(b_sf + 8 * (k & 3), (k >> 2) & 1);
             if (!ok) break;
@@ -317,12 +320,13 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
                 for (; issued < issued_after(k); ++issued) issue(issued);
             }
         }
-        if (!ok && inputs && lane == 0) atomicExch(err, kErrWaitTimeout);  // a label never arrived
-        if ((!ok || !sums) && inputs && lane == 0) {
-            // the copies in flight land before the block's shared memory goes,
-            // whatever becomes of the labels
-            issued = min(issued, il + 1);
-            for (int i = max(0, issued - kAux); i < issued; ++i)
+        if (!ok && sums && lane == 0) {
+            // a label never arrived (one that gives up does not): report it and
+            // let the copies in flight land before the block's shared memory
+            // goes; the rows issued by then follow from the step
+            atomicExch(err, kErrWaitTimeout);
+            const int n = min(k > 0 ? issued_after(k - 1) : kState, il + 1);
+            for (int i = max(0, n - kAux); i < n; ++i)
                 mbar_wait(b_full + 8 * (i & (kAux - 1)), (i / kAux) & 1);
         }
         return;

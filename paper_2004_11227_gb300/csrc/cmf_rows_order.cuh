@@ -31,10 +31,10 @@ CMF_ORDER int service_warps(int T, int LC) { return T == 2 && LC > 4 ? 2 : 1; }
 CMF_ORDER int issued_after(int k) { return k + 3 + kState; }
 // Whether a label waits for an input row (k + 2) at step k; il: the last row.
 CMF_ORDER bool label_waits_row(int k, int il) { return k + 2 <= il; }
-// Whether a service warp without the sums still waits for the labels' steps: not
-// once its rows are issued, for from then on no label waits for it, and one that
-// came late would find those steps' barriers used again.
-CMF_ORDER bool inputs_wait(int issued, int il) { return issued <= il; }
+// The last step of the labels that a service warp without the sums waits for: the
+// one behind which it issues its last row.  From then on no label waits for it, and
+// if it came late it would find the barriers of later steps used again.
+CMF_ORDER int last_input_step(int il) { return il > 2 + kState ? il - 2 - kState : 0; }
 
 }  // namespace rows
 }  // namespace cmf

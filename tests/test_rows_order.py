@@ -24,7 +24,7 @@ int ps_rows() { return rows::kPs; }
 int service_warps(int T, int LC) { return rows::service_warps(T, LC); }
 int issued_after(int k) { return rows::issued_after(k); }
 int label_waits_row(int k, int il) { return rows::label_waits_row(k, il); }
-int inputs_wait(int issued, int il) { return rows::inputs_wait(issued, il); }
+int last_input_step(int il) { return rows::last_input_step(il); }
 }
 """
 
@@ -108,9 +108,7 @@ def admm_rows(o, T, LC, L, n, rng, slow, weight):
             issue(issued)
             issued += 1
             yield None
-        for k in range(ke + 1):
-            if not sums and not o.inputs_wait(issued, il):
-                break
+        for k in range((ke if sums else o.last_input_step(il)) + 1):
             yield sf[k & 3], (k >> 2) & 1
             if sums:
                 p_s = aux[(k + 1) % kA]  # of a row behind the last one: not used
@@ -127,9 +125,6 @@ def admm_rows(o, T, LC, L, n, rng, slow, weight):
                 issue(issued)
                 issued += 1
                 yield None
-        if inputs and not sums:  # its copies land
-            for i in range(max(0, min(issued, il + 1) - kA), min(issued, il + 1)):
-                yield full[i % kA], (i // kA) & 1
 
     def label(l):
         for i in (0, 1):
