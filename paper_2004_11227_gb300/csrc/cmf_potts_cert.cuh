@@ -14,7 +14,7 @@
 // rf + k; a label reads row k + 1 of the state, row k's costs, p_s and alpha.
 //   - row k + kRing is issued when every label has done step k: its state slot
 //     was read in step k - 1, its cost slot in step k, and its threshold slot
-//     with the state;
+//     with the state (row 0's before the first step, see cmf_rows_order.cuh);
 //   - a candidate slot is rewritten kRing steps on, after its writer has had a
 //     row that was issued after the sum over that slot.
 //
@@ -34,8 +34,6 @@
 namespace cmf {
 namespace cert {
 
-constexpr int kRing = 8;
-
 template <int LC, int ES>
 struct Layout {
     static constexpr int fs = rows::up128(LC * rows::Seg<ES>::cols * ES);
@@ -51,8 +49,6 @@ struct Layout {
     static constexpr int o_bar = o_us + kRing * 256;
     static constexpr int bytes = o_bar + 3 * 8 * kRing + 128;
 };
-
-constexpr int theta_warps(int LC) { return LC / 4; }
 
 }  // namespace cert
 
@@ -137,6 +133,7 @@ __global__ void __launch_bounds__(32 * (LC + cert::theta_warps(LC) + 1),
         Row<S> x0, x1;
         float2 th0 = make_float2(0.f, 0.f), fy_up = th0, py_up = th0;
         ok = mbar_wait(b_full, 0);
+        if (cert::thresholds_from(0) == 0) ok = ok && mbar_wait(b_th, 0);
         if (ok) load_row(0, x1);
 #pragma unroll 1
         for (int k = 0; ok && k <= ke; ++k) {

@@ -37,4 +37,18 @@ CMF_ORDER bool label_waits_row(int k, int il) { return k + 2 <= il; }
 CMF_ORDER int last_input_step(int il) { return il > 2 + kState ? il - 2 - kState : 0; }
 
 }  // namespace rows
+
+namespace cert {
+
+constexpr int kRing = 8;  // rows of every kind in shared memory
+
+// Warps that find the simplex thresholds, rows in turn.
+CMF_ORDER int theta_warps(int LC) { return LC / 4; }
+// A label waits before step k for the thresholds of rows thresholds_from(k) to
+// k + 1: of row 0 too, which it does not use, for row kRing is issued into row 0's
+// slot when every label is done with step 0, and the warp that finds row 0's
+// thresholds has to have read that row by then.
+CMF_ORDER int thresholds_from(int k) { return k == 0 ? 0 : k + 1; }
+
+}  // namespace cert
 }  // namespace cmf

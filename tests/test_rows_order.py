@@ -25,6 +25,9 @@ int service_warps(int T, int LC) { return rows::service_warps(T, LC); }
 int issued_after(int k) { return rows::issued_after(k); }
 int label_waits_row(int k, int il) { return rows::label_waits_row(k, il); }
 int last_input_step(int il) { return rows::last_input_step(il); }
+int cert_ring() { return cert::kRing; }
+int theta_warps(int LC) { return cert::theta_warps(LC); }
+int thresholds_from(int k) { return cert::thresholds_from(k); }
 }
 """
 
@@ -160,4 +163,71 @@ def test_admm_rows_never_stuck(order, T, LC, L, weight):
         for slow in range(L + 3):
             for seed in range(3):
                 assert admm_rows(order, T, LC, L, n, random.Random(seed), slow, weight), \
+                    (n, slow, seed)
+
+
+def certificate_rows(o, LC, L, n, rng, slow, weight):
+    """k_potts_cert: a band of n rows, L labels in a class of LC."""
+    R, NT = o.cert_ring(), o.theta_warps(LC)
+    il, ke = n + 1, n
+    full, th = [Bar(1) for _ in range(R)], [Bar(1) for _ in range(R)]
+    sf = [Bar(L) for _ in range(R)]
+    rows, thr, flight = [None] * R, [None] * R, []
+    shares = [[None] * L for _ in range(R)]
+
+    def issue(i):
+        if i <= il:
+            rows[i % R] = "in flight"
+            flight.append(i)
+
+    def land(i):
+        rows[i % R] = i
+        full[i % R].arrive()
+
+    def label(l):
+        yield full[0], 0
+        for i in range(o.thresholds_from(0), 1):
+            yield th[i], 0
+        assert rows[0] == 0
+        for k in range(ke + 1):
+            yield full[(k + 1) % R], (k + 1) // R & 1
+            for i in range(max(1, o.thresholds_from(k)), k + 2):
+                yield th[i % R], i // R & 1
+            assert rows[(k + 1) % R] == k + 1 and rows[k % R] == k and thr[(k + 1) % R] == k + 1
+            yield None
+            assert rows[(k + 1) % R] == k + 1 and rows[k % R] == k and thr[(k + 1) % R] == k + 1
+            shares[k % R][l] = k
+            yield None
+            sf[k % R].arrive()
+
+    def theta(w):
+        for i in range(w, il + 1, NT):
+            yield full[i % R], i // R & 1
+            for _ in range(3):
+                assert rows[i % R] == i, "overwritten while read"
+                yield None
+            thr[i % R] = i
+            th[i % R].arrive()
+
+    def last():
+        for i in range(R):
+            issue(i)
+            yield None
+        for k in range(ke + 1):
+            yield sf[k % R], k // R & 1
+            assert shares[k % R] == [k] * L
+            yield None
+            issue(k + R)
+
+    tasks = [label(l) for l in range(L)] + [theta(w) for w in range(NT)] + [last()]
+    return replay(tasks, flight, land, rng, slow % (len(tasks) + 1), weight)
+
+
+@pytest.mark.parametrize("weight", [1.0, 0.1, 0.01, 0.001])
+@pytest.mark.parametrize("LC,L", [(4, 3), (8, 5), (16, 9)])
+def test_certificate_rows_never_stuck(order, LC, L, weight):
+    for n in (1, 2, 6, 7, 8, 9, 20):
+        for slow in range(L + LC // 4 + 2):
+            for seed in range(3):
+                assert certificate_rows(order, LC, L, n, random.Random(seed), slow, weight), \
                     (n, slow, seed)
