@@ -641,9 +641,13 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         }
         return e;
     };
+    // the results, on the call's own stream
     auto collect = [&]() -> cmf_status {
         int herr = 0;
-        CMF_CUDA_TRY(cudaMemcpy(&herr, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost));
+        CMF_CUDA_TRY(cudaMemcpyAsync(&herr, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CMF_CUDA_TRY(cudaMemcpyAsync(desc.data(), d_desc, sizeof(BatchDesc) * n,
+                                     cudaMemcpyDeviceToHost, st));
+        CMF_CUDA_TRY(cudaStreamSynchronize(st));
         if (herr == kErrWaitTimeout) return CMF_ETIMEOUT;
         bool all_ok = true;
         for (int i = 0; i < n; ++i) {
@@ -666,9 +670,6 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             CMF_CUDA_TRY(cudaStreamSynchronize(st));
             if (hc.stop) break;
         }
-        CMF_CUDA_TRY(cudaMemcpyAsync(desc.data(), d_desc, sizeof(BatchDesc) * n,
-                                     cudaMemcpyDeviceToHost, st));
-        CMF_CUDA_TRY(cudaStreamSynchronize(st));
         return collect();
     }
 
@@ -712,10 +713,6 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         if (e != cudaSuccess || e2 != cudaSuccess) break;
         if (cudaGraphInstantiate(&ge, g, 0) != cudaSuccess) break;
         if (cudaGraphLaunch(ge, st) != cudaSuccess) break;
-        if (cudaMemcpyAsync(desc.data(), d_desc, sizeof(BatchDesc) * n, cudaMemcpyDeviceToHost,
-                            st) != cudaSuccess)
-            break;
-        if (cudaStreamSynchronize(st) != cudaSuccess) break;
         status = collect();
     } while (0);
     if (ge) cudaGraphExecDestroy(ge);
