@@ -3,8 +3,8 @@
 The translation units are compiled in parallel and linked into
 ``paper_2004_11227_gb300/libcmf.so``; objects go to ``paper_2004_11227_gb300/_build``.
 The same batch builds ``libcmf_inject.so``, the fault-injection library of
-the failure-detection tests: the translation units with bounded device waits
-compiled again with CMF_FAULT_INJECTION (a short wait limit and a hook that
+the failure-detection tests: translation units with bounded device waits (those
+of the automatic choice in float32 storage, and the TMA tiles') compiled again with CMF_FAULT_INJECTION (a short wait limit and a hook that
 makes a wait run out), linked with the other objects.  Nothing on the product
 path loads it.
 """
@@ -21,8 +21,11 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcmf.so")
 LIB_INJECT = os.path.join(PKG, "libcmf_inject.so")
-# translation units with bounded device waits (rebuilt for the injection library)
-INJECT_TUS = ("cmf_binary_tma.cu", "cmf_potts_tma.cu")
+# translation units with bounded device waits, rebuilt for the injection library (the
+# 16-bit and odd-width instantiations of the same kernels are not)
+INJECT_TUS = ("cmf_binary_tma.cu", "cmf_potts_tma.cu", "cmf_potts_rows_f32.cu",
+              "cmf_potts_cert_f32.cu", "cmf_potts_dr_rows_f32.cu", "cmf_binary_chain_f32.cu",
+              "cmf_binary_dr_rows.cu", "cmf_batch_rows_f32.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

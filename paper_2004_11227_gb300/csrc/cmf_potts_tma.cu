@@ -404,4 +404,11 @@ extern "C" cmf_status cmf_debug_inject_tx_mismatch(unsigned int bytes) {
                ? CMF_OK
                : CMF_ECUDA;
 }
+// The same for every barrier that waits for input rows, in all the units built for
+// injection (the kernels of the automatic choice in float32 storage).
+extern "C" cmf_status cmf_debug_inject_row_tx(unsigned int bytes) {
+    for (auto hook : cmf::inject_hooks())
+        if (hook(bytes) != cudaSuccess) return CMF_ECUDA;
+    return CMF_OK;
+}
 #endif

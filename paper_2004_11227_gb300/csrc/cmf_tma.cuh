@@ -7,7 +7,31 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#ifdef CMF_FAULT_INJECTION
+#include <vector>
+#endif
+
 namespace cmf {
+
+#ifdef CMF_FAULT_INJECTION
+// Fault-injection test build only (never in the library the product loads):
+// extra bytes every row barrier of this translation unit expects beyond what its
+// copies deliver.  With a non-zero value no such phase can complete, the bounded
+// waits run out, and the kernels record kErrWaitTimeout and return; nothing
+// faults and no copy is left in flight.
+static __device__ unsigned int g_inject_row_tx = 0;
+static cudaError_t inject_row_tx(unsigned int bytes) {
+    return cudaMemcpyToSymbol(g_inject_row_tx, &bytes, sizeof(bytes));
+}
+inline std::vector<cudaError_t (*)(unsigned int)>& inject_hooks() {  // one per unit
+    static std::vector<cudaError_t (*)(unsigned int)> hooks;
+    return hooks;
+}
+static const bool g_inject_hooked = (inject_hooks().push_back(inject_row_tx), true);
+#define CMF_ROW_EXTRA_TX g_inject_row_tx
+#else
+#define CMF_ROW_EXTRA_TX 0u
+#endif
 
 // ---- device side -----------------------------------------------------------
 
@@ -33,7 +57,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
+                 "r"(bytes + CMF_ROW_EXTRA_TX)
                  : "memory");
 }
 
