@@ -422,7 +422,8 @@ typedef struct {
     void *d_ps;             /* p_s (1 plane; Potts: float32)                    */
     /* results (outputs) */
     int iters;              /* iterations run for this instance                 */
-    int status;             /* CMF_OK or CMF_NOT_CONVERGED                      */
+    int status;             /* CMF_OK or CMF_NOT_CONVERGED; CMF_ETIMEOUT: still
+                               iterating when a device-side wait ran out        */
     double energy, dual, gap, res;  /* last certificates (as cmf_eval_*)       */
 } cmf_instance;
 
@@ -441,7 +442,8 @@ size_t cmf_batch_workspace_bytes(const cmf_instance *inst, int n, const cmf_para
  * cold start unless p->warm_start.  Fills the
  * result fields of every instance.  Returns CMF_OK when every instance
  * reached p->tol_gap, CMF_NOT_CONVERGED when some stopped at max_iter,
- * CMF_ETIMEOUT when a bounded device-side wait ran out. */
+ * CMF_ETIMEOUT when a bounded device-side wait ran out (the batch then stops at
+ * its next check). */
 cmf_status cmf_solve_batch(cmf_instance *inst, int n, const cmf_params *p, void *d_ws,
                            size_t ws_bytes, void *stream);
 

@@ -276,12 +276,14 @@ __global__ void k_batch_reduce(const BatchDesc* desc, const double* partials, do
     }
 }
 
-// One block: retire converged instances, decide whether the loop runs again.
+// One block: retire converged instances, decide whether the loop runs again.  A
+// device wait that ran out retires all of them: their states are undefined.
 // set_h = 0: a host-driven loop (no graph), which reads ctl->stop instead.
 __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, BatchCtl* ctl, int K,
                                int max_iter, double tol, MergeRule rule,
                                cudaGraphConditionalHandle h, int set_h) {
     const int it = ctl->it + K;
+    const bool failed = ctl->err == kErrWaitTimeout;
     int any = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         BatchDesc& D = desc[i];
@@ -293,7 +295,10 @@ __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, Batch
         D.dual = Dv;
         D.gap = gap;
         D.res = sqrt(R > 0.0 ? R : 0.0);
-        if (gap <= tol) {
+        if (failed) {
+            D.active = 0;
+            D.status = CMF_ETIMEOUT;
+        } else if (gap <= tol) {
             D.active = 0;
             D.status = CMF_OK;
         } else if (it + K > max_iter) {
@@ -648,7 +653,6 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         CMF_CUDA_TRY(cudaMemcpyAsync(desc.data(), d_desc, sizeof(BatchDesc) * n,
                                      cudaMemcpyDeviceToHost, st));
         CMF_CUDA_TRY(cudaStreamSynchronize(st));
-        if (herr == kErrWaitTimeout) return CMF_ETIMEOUT;
         bool all_ok = true;
         for (int i = 0; i < n; ++i) {
             inst[i].iters = desc[i].iters;
@@ -659,6 +663,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             inst[i].res = desc[i].res;
             all_ok = all_ok && desc[i].status == CMF_OK;
         }
+        if (herr == kErrWaitTimeout) return CMF_ETIMEOUT;
         return all_ok ? CMF_OK : CMF_NOT_CONVERGED;
     };
     if (!p->use_graph) {

@@ -1,7 +1,7 @@
-"""A bounded wait that runs out in a kernel of the automatic choice is reported as
-CMF_ETIMEOUT, stops the solve at its next check and leaves the context usable: the
-fault-injection library (see test_gpu_failure.py) makes every barrier that waits for
-input rows expect 16 bytes more than its copies deliver."""
+"""A bounded wait that runs out in a kernel of the automatic choice, or in a batch, is
+reported as CMF_ETIMEOUT, stops the solve at its next check and leaves the context
+usable: the fault-injection library (see test_gpu_failure.py) makes every barrier that
+waits for input rows expect 16 bytes more than its copies deliver."""
 import json
 import os
 import subprocess
@@ -73,6 +73,25 @@ for name, args in CASES.items():
     after = q.solve()
     r["after_equal"] = after == before
     out[name] = r
+
+for use_graph in (1, 0):
+    p = cmf.default_params(2, 2, tol_gap=1e-3, max_iter=10000000, check_every=10,
+                           use_graph=use_graph)
+    items = [cmf.alloc_binary(synth.random_binary(40, 60, seed=1), p)]
+    items += [cmf.alloc_potts(synth.random_potts(33 + L, 50 + L, L, seed=L), p)
+              for L in (3, 4, 7, 12)]
+    b = cmf.Batch(items, p)
+    def run():
+        st = lib.cmf_solve_batch(b.insts, len(items), ctypes.byref(p), cmf._ptr(b.ws),
+                                 b.ws.numel(), cmf._stream(None))
+        return [st] + [[d.status, d.iters, d.gap] for d in b.insts]
+    before = run()
+    inject(16)
+    failed = run()
+    inject(0)
+    out[f"batch_{use_graph}"] = {"before": before[0], "solve": failed[0],
+                                 "items": [x[:2] for x in failed[1:]],
+                                 "after_equal": run() == before}
 torch.cuda.synchronize()
 print("RESULT " + json.dumps(out))
 """
@@ -96,6 +115,7 @@ def result():
 
     __graft_entry__.build()
     code = f"ROOT = {ROOT!r}\nCASES = {CASES!r}\n" + CHILD
+    # a batch that ran on to its iteration limit would take hours
     proc = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
                           timeout=600)
     assert proc.returncode == 0, proc.stderr[-3000:]
@@ -113,3 +133,11 @@ def test_default_kernels_report_a_timeout(result, case):
     assert r["iterate"] == OK and r["evals"] == [ETIMEOUT, OK]
     assert r.get("eval_itself", ETIMEOUT) == ETIMEOUT
     assert r["after_equal"]  # the same history bit for bit
+
+
+@pytest.mark.parametrize("use_graph", [1, 0])
+def test_batch_stops_at_its_next_check(result, use_graph):
+    r = result[f"batch_{use_graph}"]
+    assert r["before"] == OK and r["solve"] == ETIMEOUT
+    assert r["items"] == [[ETIMEOUT, 10]] * 5
+    assert r["after_equal"]
