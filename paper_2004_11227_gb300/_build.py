@@ -21,9 +21,10 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcmf.so")
 LIB_INJECT = os.path.join(PKG, "libcmf_inject.so")
-# translation units with bounded device waits, rebuilt for the injection library (the
-# 16-bit and odd-width instantiations of the same kernels are not)
-INJECT_TUS = ("cmf_binary_tma.cu", "cmf_potts_tma.cu", "cmf_potts_rows_f32.cu",
+# translation units rebuilt for the injection library: with bounded device waits (the
+# 16-bit and odd-width instantiations of the same kernels are not), and the tensor maps'
+# (a count of the encodings)
+INJECT_TUS = ("cmf_tma.cu", "cmf_binary_tma.cu", "cmf_potts_tma.cu", "cmf_potts_rows_f32.cu",
               "cmf_potts_cert_f32.cu", "cmf_potts_dr_rows_f32.cu", "cmf_binary_chain_f32.cu",
               "cmf_binary_dr_rows.cu", "cmf_batch_rows_f32.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -213,7 +213,10 @@ struct BinaryCall {
     bool pairs;             // warp strips, two ADMM iterations per launch
     bool chain;             // chains of warps, up to four ADMM iterations per launch
     bool dr_rows;           // rPDRQ on shared TMA rows
-    BinChainMaps cmaps[3];  // tensor maps of the buffer sets
+    // tensor maps of the buffer sets (chain, dr_rows), encoded by binary_maps
+    // where a launch first reads a set
+    mutable BinChainMaps cmaps[3];
+    mutable int mapped = 0;  // the sets encoded, a bit each
     int cert_blocks;        // partial triples the workspace holds
     BinTmaMaps maps[2];     // tensor maps of the user / workspace state sets
     int* err;               // sticky device error word
@@ -258,9 +261,7 @@ cmf_status binary_prepare(const float* Cs, const float* Ct, const float* alpha, 
     if (!call.cfg.plain && !call.cfg.dr &&
         (p->variant == 0 || (p->variant == 4 && W % 2 == 0)) &&
         binary_chain_eligible(call.P, p->storage, call.user, call.ws, call.ws2) &&
-        binary_chain_maps(call.P, p->storage, call.user, call.cmaps[0]) == cudaSuccess &&
-        binary_chain_maps(call.P, p->storage, call.ws, call.cmaps[1]) == cudaSuccess &&
-        binary_chain_maps(call.P, p->storage, call.ws2, call.cmaps[2]) == cudaSuccess) {
+        tma_available()) {
         call.chain = true;
         const int nb = eval_blocks(H, W), nc = binary_cert_max_blocks();
         call.cert_blocks = nb > nc ? nb : nc;
@@ -271,8 +272,7 @@ cmf_status binary_prepare(const float* Cs, const float* Ct, const float* alpha, 
     // per iteration, with the same results)
     if (!call.cfg.plain && call.cfg.dr && p->variant == 0 &&
         binary_dr_rows_eligible(call.P, p->storage, call.cfg.dc, call.user, call.ws) &&
-        binary_dr_rows_maps(call.P, p->storage, call.user, call.cmaps[0]) == cudaSuccess &&
-        binary_dr_rows_maps(call.P, p->storage, call.ws, call.cmaps[1]) == cudaSuccess) {
+        tma_available()) {
         call.dr_rows = true;
         return CMF_OK;
     }
@@ -309,6 +309,21 @@ cmf_status binary_prepare(const float* Cs, const float* Ct, const float* alpha, 
 
 const BinStateV& bset(const BinaryCall& c, int i) {
     return i == 0 ? c.user : (i == 1 ? c.ws : c.ws2);
+}
+
+// The tensor maps of buffer set i.  All three sets' (24 driver calls, 3.5 us of a
+// 50 us certificate call at 64^2) are seldom read: certificates and replayed graphs
+// read none, one iteration reads the caller's.
+cudaError_t binary_maps(const BinaryCall& c, int i) {
+    if (c.mapped >> i & 1) return cudaSuccess;
+    const BinChainMaps* planes = nullptr;  // of a set already encoded
+    for (int k = 0; k < 3; ++k)
+        if (c.mapped >> k & 1) planes = &c.cmaps[k];
+    const cudaError_t e =
+        c.chain ? binary_chain_maps(c.P, c.storage, bset(c, i), c.cmaps[i], planes)
+                : binary_dr_rows_maps(c.P, c.storage, bset(c, i), c.cmaps[i], planes);
+    if (e == cudaSuccess) c.mapped |= 1 << i;
+    return e;
 }
 
 // Run n iterations starting from `cur` (0 = user buffers, 1 = workspace,
@@ -351,9 +366,11 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
             certified = may_cert && j == first + nl - 1;
             if (!dry) {
                 const StepConfig cfg = m < 0 ? step_at(c.cfg, c.prm, 2, false, k0 + j) : c.cfg;
-                cudaError_t e = binary_chain_step(c.storage, c.P, bset(c, dst), cfg.aniso, cfg.ac,
-                                                  T, i, c.cmaps[cur], partials, c.cert_blocks,
-                                                  certified ? cert : nullptr, c.err, st);
+                cudaError_t e = binary_maps(c, cur);
+                if (e == cudaSuccess)
+                    e = binary_chain_step(c.storage, c.P, bset(c, dst), cfg.aniso, cfg.ac, T, i,
+                                          c.cmaps[cur], partials, c.cert_blocks,
+                                          certified ? cert : nullptr, c.err, st);
                 if (e != cudaSuccess) return e;
             }
             if (m >= 0) i += T;
@@ -408,8 +425,10 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
             cur = 0;
         } else if (c.dr_rows) {
             if (!dry) {
-                cudaError_t e = binary_dr_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user,
-                                                    cfg.aniso, cfg.dc, c.cmaps[cur], c.err, st);
+                cudaError_t e = binary_maps(c, cur);
+                if (e == cudaSuccess)
+                    e = binary_dr_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso,
+                                            cfg.dc, c.cmaps[cur], c.err, st);
                 if (e != cudaSuccess) return e;
             }
             cur ^= 1;
@@ -537,19 +556,20 @@ struct PottsCall {
     bool cert;                   // certificates with the labels side by side
     bool dr_rows;                // rPDRQ with the labels side by side
     PottsTmaMaps maps[2];        // tensor maps of the user / workspace state sets
-    PottsRowsMaps rmaps[2];
+    // tensor maps of the two sets (rows, dr_rows, cert), encoded by row_maps
+    // where a launch first reads a set
+    mutable PottsRowsMaps rmaps[2];
+    mutable int mapped = 0;  // the sets encoded, a bit each
     int rfused;                  // potts_rows_fused
     int* err;                    // sticky device error word
 };
 
 // `layout`: the parameters the workspace was sized for (default *p); `set`:
-// the second state set (default: the workspace's own, in p->storage); `certs`:
-// whether certificates may follow.
+// the second state set (default: the workspace's own, in p->storage).
 cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0, int H, int W,
                          int pitch, const cmf_params* p, float* u, void* qx, void* qy, void* pp,
                          void* ps, void* ws, size_t ws_bytes, PottsCall& call,
-                         const cmf_params* layout = nullptr, const PottsStateV* set = nullptr,
-                         bool certs = true) {
+                         const cmf_params* layout = nullptr, const PottsStateV* set = nullptr) {
     cmf_status s;
     if (L < 2 || L > 64) return CMF_EINVAL;
     if ((s = check_params(p, L)) != CMF_OK) return s;
@@ -587,11 +607,7 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     const bool rows =
         free_choice && !call.cfg.dr &&
         potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws);
-    // the maps: fourteen driver calls, about 4 us, only where a launch reads them
-    call.cert = (certs || rows || dr_rows) &&
-                potts_rows_layout(call.P, p->storage, call.user, call.ws) &&
-                potts_rows_maps(call.P, p->storage, call.user, call.rmaps[0]) == cudaSuccess &&
-                potts_rows_maps(call.P, p->storage, call.ws, call.rmaps[1]) == cudaSuccess;
+    call.cert = potts_rows_layout(call.P, p->storage, call.user, call.ws) && tma_available();
     if (dr_rows && call.cert) {
         call.dr_rows = true;
         return CMF_OK;
@@ -626,15 +642,28 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     return CMF_OK;
 }
 
+// The tensor maps of buffer set i (as binary_maps: most calls read one set's or
+// none).
+cudaError_t row_maps(const PottsCall& c, int i) {
+    if (c.mapped >> i & 1) return cudaSuccess;
+    const cudaError_t e = potts_rows_maps(c.P, c.storage, i == 0 ? c.user : c.ws, c.rmaps[i],
+                                          c.mapped ? &c.rmaps[i ^ 1] : nullptr);
+    if (e == cudaSuccess) c.mapped |= 1 << i;
+    return e;
+}
+
 // The certificate launch for buffer set `set` (0 or 1): labels side by side
 // where the layout allows it (a call, host part included: 2048^2, L = 16
 // 547 -> 423 us, L = 4 197 -> 153 us; 721 x 1283, L = 8 199 -> 97 us; not
 // slower anywhere from 128^2 on), else the strip or tile kernel.
 cudaError_t potts_certify(const PottsCall& c, int set, cudaStream_t st, const EvalTail& T) {
     double* partials = (double*)(c.wsbase + c.w.partials);
-    if (c.cert)
+    if (c.cert) {
+        const cudaError_t e = row_maps(c, set);
+        if (e != cudaSuccess) return e;
         return potts_cert(c.storage, c.P, c.rmaps[set], c.cfg.aniso, c.cfg.dr, c.cfg.dc.tau,
                           partials, T, c.err, st);
+    }
     return potts_eval(c.storage, c.P, set == 0 ? c.user : c.ws, c.cfg.aniso, c.cfg.dr,
                       c.cfg.dc.tau, partials, st, T);
 }
@@ -656,9 +685,10 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
             const int it = i < singles ? 1 : 2;
             if (!dry) {
                 const StepConfig cfg = step_at(c.cfg, c.prm, c.P.L, true, k0 + i);
-                cudaError_t e =
-                    potts_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso, cfg.ac,
-                                    cu_in, it, c.rmaps[cur], c.rfused, c.err, st);
+                cudaError_t e = row_maps(c, cur);
+                if (e == cudaSuccess)
+                    e = potts_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso,
+                                        cfg.ac, cu_in, it, c.rmaps[cur], c.rfused, c.err, st);
                 if (e != cudaSuccess) return e;
             }
             cu_in = c.cfg.ac.cu;
@@ -684,8 +714,10 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
             if (e != cudaSuccess) return e;
             cur = 0;
         } else if (c.dr_rows) {
-            cudaError_t e = potts_dr_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user,
-                                               cfg.aniso, cfg.dc, c.rmaps[cur], c.err, st);
+            cudaError_t e = row_maps(c, cur);
+            if (e == cudaSuccess)
+                e = potts_dr_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso,
+                                       cfg.dc, c.rmaps[cur], c.err, st);
             if (e != cudaSuccess) return e;
             cur ^= 1;
         } else if (c.strip && cfg.dr) {
@@ -1300,7 +1332,7 @@ cmf_status cmf_iterate_potts(const float* d_C, int L, const float* d_alpha, floa
                              size_t ws_bytes, void* stream) {
     PottsCall c;
     cmf_status s = potts_prepare(d_C, L, d_alpha, alpha0, H, W, pitch, p, d_u, d_qx, d_qy, d_p,
-                                 d_ps, d_ws, ws_bytes, c, nullptr, nullptr, false);
+                                 d_ps, d_ws, ws_bytes, c);
     if (s != CMF_OK) return s;
     if (n_iter < 0) return CMF_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;

@@ -40,24 +40,30 @@ bool binary_chain_certifies(const Grid& G, int max_blocks) {
 }
 
 cudaError_t binary_chain_maps(const BinProblem& P, int storage, const BinStateV& s,
-                              BinChainMaps& m) {
+                              BinChainMaps& m, const BinChainMaps* planes) {
     return binary_row_maps(
         P, storage, s, dtype_size(storage) == 4 ? chain::Seg<4>::cols : chain::Seg<2>::cols,
-        chain::Seg<4>::cols, m);
+        chain::Seg<4>::cols, m, planes);
 }
 
 cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s, int cs, int c4,
-                            BinChainMaps& m) {
+                            BinChainMaps& m, const BinChainMaps* planes) {
     const Grid& G = P.g;
     const int es = (int)dtype_size(storage);
     const struct {
         CUtensorMap* map;
         const void* base;
         int es, box;
-    } f[8] = {{&m.qx, s.qx, es, cs}, {&m.qy, s.qy, es, cs}, {&m.ps, s.ps, es, cs},
+    } f[] = {{&m.qx, s.qx, es, cs}, {&m.qy, s.qy, es, cs}, {&m.ps, s.ps, es, cs},
               {&m.pt, s.pt, es, cs}, {&m.u, s.u, 4, c4},    {&m.Cs, P.Cs, 4, c4},
               {&m.Ct, P.Ct, 4, c4},  {&m.al, P.alpha.plane, 4, c4}};
     for (const auto& q : f) {
+        if (planes && q.map == &m.Cs) {
+            m.Cs = planes->Cs;
+            m.Ct = planes->Ct;
+            m.al = planes->al;
+            break;
+        }
         if (!q.base) {  // constant alpha: its map is never read
             *q.map = m.u;
             continue;

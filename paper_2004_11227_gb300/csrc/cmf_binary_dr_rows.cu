@@ -318,10 +318,10 @@ bool binary_dr_rows_eligible(const BinProblem& P, int storage, const DrCoef& D,
 }
 
 cudaError_t binary_dr_rows_maps(const BinProblem& P, int storage, const BinStateV& s,
-                                BinChainMaps& m) {
+                                BinChainMaps& m, const BinChainMaps* planes) {
     const int es = (int)dtype_size(storage);
     return binary_row_maps(P, storage, s, es == 4 ? bdr::Seg<4>::cols : bdr::Seg<2>::cols,
-                           bdr::Seg<4>::cols, m);
+                           bdr::Seg<4>::cols, m, planes);
 }
 
 cudaError_t binary_dr_rows_step(int storage, const BinProblem& P, const BinStateV& b, bool aniso,

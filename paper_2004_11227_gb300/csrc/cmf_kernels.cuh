@@ -381,8 +381,10 @@ bool binary_chain_eligible(const BinProblem& P, int storage, const BinStateV& a,
                            const BinStateV& b, const BinStateV& c);
 // Whether a launch can certify its result with at most max_blocks partials.
 bool binary_chain_certifies(const Grid& G, int max_blocks);
+// planes: the maps of another state of the same problem (its cost and alpha planes'
+// maps are copied).
 cudaError_t binary_chain_maps(const BinProblem& P, int storage, const BinStateV& s,
-                              BinChainMaps& m);
+                              BinChainMaps& m, const BinChainMaps* planes = nullptr);
 // T iterations (1 .. binary_chain_max_iters) from the state of src_maps into
 // b; iter0: the first one's index among the call's unscheduled iterations;
 // cert: as binary_strip2_step, with at most max_blocks partial triples; a
@@ -395,7 +397,7 @@ cudaError_t binary_chain_step(
 // Maps of a state and its cost planes in boxes of one row: cs columns of the
 // stored flows, c4 of the float32 planes.
 cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s, int cs, int c4,
-                            BinChainMaps& m);
+                            BinChainMaps& m, const BinChainMaps* planes);
 
 // --- binary rPDRQ on shared TMA rows (cmf_binary_dr_rows.cu) ---
 // One iteration from the state of src_maps into b; a bounded wait that runs out
@@ -403,7 +405,7 @@ cudaError_t binary_row_maps(const BinProblem& P, int storage, const BinStateV& s
 bool binary_dr_rows_eligible(const BinProblem& P, int storage, const DrCoef& D,
                              const BinStateV& a, const BinStateV& b);
 cudaError_t binary_dr_rows_maps(const BinProblem& P, int storage, const BinStateV& s,
-                                BinChainMaps& m);
+                                BinChainMaps& m, const BinChainMaps* planes = nullptr);
 cudaError_t binary_dr_rows_step(int storage, const BinProblem& P, const BinStateV& b, bool aniso,
                                 const DrCoef& D, const BinChainMaps& src_maps, int* err,
                                 cudaStream_t st);
@@ -450,7 +452,7 @@ bool potts_rows_eligible(const PottsProblem& P, int storage, const AdmmCoef& K,
 // 16-row instantiations do, its 8-row ones do not) rounds products into sums.
 int potts_rows_fused(const PottsProblem& P, int storage, bool aniso);
 cudaError_t potts_rows_maps(const PottsProblem& P, int storage, const PottsStateV& s,
-                            PottsRowsMaps& m);
+                            PottsRowsMaps& m, const PottsRowsMaps* planes = nullptr);
 // `iters` (1 or 2) iterations from the state of src_maps into b, with the
 // multiplier form of potts_strip_step; a bounded wait that runs out sets *err.
 cudaError_t potts_rows_step(int storage, const PottsProblem& P, const PottsStateV& b, bool aniso,

@@ -72,7 +72,7 @@ int potts_rows_fused(const PottsProblem& P, int storage, bool aniso) {
 }
 
 cudaError_t potts_rows_maps(const PottsProblem& P, int storage, const PottsStateV& s,
-                            PottsRowsMaps& m) {
+                            PottsRowsMaps& m, const PottsRowsMaps* planes) {
     const Grid& G = P.g;
     const int es = (int)dtype_size(storage);
     const int cs = es == 4 ? rows::Seg<4>::cols : rows::Seg<2>::cols, c4 = rows::Seg<4>::cols;
@@ -80,10 +80,15 @@ cudaError_t potts_rows_maps(const PottsProblem& P, int storage, const PottsState
         CUtensorMap* map;
         const void* base;
         int es, planes, box;
-    } f[7] = {{&m.qx, s.qx, es, P.L, cs}, {&m.qy, s.qy, es, P.L, cs}, {&m.p, s.p, es, P.L, cs},
+    } f[] = {{&m.qx, s.qx, es, P.L, cs}, {&m.qy, s.qy, es, P.L, cs}, {&m.p, s.p, es, P.L, cs},
               {&m.u, s.u, 4, P.L, c4},    {&m.ps, s.ps, 4, 1, c4},    {&m.C, P.C, 4, P.L, c4},
               {&m.al, P.alpha.plane, 4, 1, c4}};
     for (const auto& q : f) {
+        if (planes && q.map == &m.C) {
+            m.C = planes->C;
+            m.al = planes->al;
+            break;
+        }
         if (!q.base) {  // constant alpha: its map is never read
             *q.map = m.ps;
             continue;

@@ -119,6 +119,9 @@ constexpr long long kWaitLimitCycles = 2000000000ll;
 
 // ---- host side -------------------------------------------------------------
 
+// Whether tensor maps can be encoded (the driver has the function).
+bool tma_available();
+
 // Encode a row-major [planes][rows][cols] tensor of `elem_bytes` elements with
 // a row stride of `pitch` elements and a plane stride of rows * pitch; box
 // {box_x, box_y, box_z}; out-of-range elements read as zero.  Returns
