@@ -120,7 +120,9 @@ typedef struct {
     int variant;       /* kernel variant of the fused ADMM algorithms:
                           0 = automatic: where rows and planes are 16-byte
                           aligned, binary: chains of warps, up to four
-                          iterations per launch; Potts with at most 16 labels
+                          iterations per launch (iterations that run alone
+                          and calls of three or four: the kernels below on
+                          grids where those are faster); Potts with at most 16 labels
                           and float32 cost planes (odd widths: rpADMMII,
                           rpADMMI, pADMMI): labels side by side, two iterations
                           per launch; rPDRQ of one sweep at even widths (Potts:

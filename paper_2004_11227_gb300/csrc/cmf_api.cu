@@ -211,6 +211,7 @@ struct BinaryCall {
     bool tma;               // fused ADMM through the persistent TMA kernel
     bool strip;             // fused ADMM by warp strips
     bool pairs;             // warp strips, two ADMM iterations per launch
+    bool alone;             // chain: iterations that run alone run by strips or TMA tiles
     bool chain;             // chains of warps, up to four ADMM iterations per launch
     bool dr_rows;           // rPDRQ on shared TMA rows
     // tensor maps of the buffer sets (chain, dr_rows), encoded by binary_maps
@@ -218,7 +219,10 @@ struct BinaryCall {
     mutable BinChainMaps cmaps[3];
     mutable int mapped = 0;  // the sets encoded, a bit each
     int cert_blocks;        // partial triples the workspace holds
-    BinTmaMaps maps[2];     // tensor maps of the user / workspace state sets
+    // tensor maps of the user / workspace state sets (tma); with chain encoded by
+    // one_iteration where a launch first reads a set
+    mutable BinTmaMaps maps[2];
+    mutable int tma_mapped = 0;  // the sets encoded, a bit each
     int* err;               // sticky device error word
 };
 
@@ -263,6 +267,21 @@ cmf_status binary_prepare(const float* Cs, const float* Ct, const float* alpha, 
         binary_chain_eligible(call.P, p->storage, call.user, call.ws, call.ws2) &&
         tma_available()) {
         call.chain = true;
+        // The iterations that run alone (a rho schedule's, a remainder) keep the
+        // kernels that made one a launch, with the same results, where a chain of
+        // one warp is slower: warp strips at even widths up to 1024^2 (512^2 8.6
+        // -> 6.5 us, 1024^2 12.7 -> 12.6; 1448^2 18.8 against 21.4) and with
+        // 16-bit flows everywhere (1024^2 13.8 -> 10.7 us, 4096^2 107 -> 101), TMA
+        // tiles at odd ones up to that size (512 x 513 8.6 -> 6.6 us, 1024 x 1025
+        // equal; 1448 x 1447 20.9 against 29.3).
+        const bool small = (size_t)H * (size_t)W <= (size_t)1 << 20;
+        call.strip = W % 2 == 0 && binary_strip_eligible(call.P.g, p->storage, Cs, Ct, alpha,
+                                                         call.user, call.ws);
+        call.alone = call.strip && (small || es == 2);
+        if (W % 2) {
+            call.tma = call.alone = small && binary_tma_eligible(call.P.g, p->storage, call.user) &&
+                                    binary_tma_eligible(call.P.g, p->storage, call.ws);
+        }
         const int nb = eval_blocks(H, W), nc = binary_cert_max_blocks();
         call.cert_blocks = nb > nc ? nb : nc;
         return CMF_OK;
@@ -326,6 +345,31 @@ cudaError_t binary_maps(const BinaryCall& c, int i) {
     return e;
 }
 
+// Whether the chain path leaves a lone iteration from set src into set dst to the
+// kernels that make one a launch: where binary_prepare chose one, among the first
+// two sets, and (iter0: its index among the call's unscheduled iterations) not
+// the second of a pair with 16-bit flows, whose roundings are the pair's.
+bool runs_alone(const BinaryCall& c, int src, int dst, int iter0) {
+    if (src > 1 || dst > 1 || !c.alone) return false;
+    return !(c.strip && c.storage != CMF_F32 && (iter0 & 1));
+}
+
+// That iteration (AdmmCoef: the scheduled one where a schedule covers it).
+cudaError_t one_iteration(const BinaryCall& c, int src, int dst, const StepConfig& cfg,
+                          cudaStream_t st) {
+    if (c.strip)
+        return binary_strip_step(c.storage, c.P, bset(c, src), bset(c, dst), cfg.aniso, cfg.ac,
+                                 st);
+    if (!(c.tma_mapped >> src & 1)) {
+        const cudaError_t e =
+            binary_tma_maps(c.P.g, c.storage, bset(c, src), 16, c.maps[src]);
+        if (e != cudaSuccess) return e;
+        c.tma_mapped |= 1 << src;
+    }
+    return binary_admm_tma_step(c.storage, c.P, bset(c, dst), cfg.aniso, cfg.ac, c.maps[src],
+                                c.err, st);
+}
+
 // Run n iterations starting from `cur` (0 = user buffers, 1 = workspace,
 // 2 = the workspace's third set, used by the two-iteration launches);
 // returns the index of the buffer set holding the result.  k0 is the index of
@@ -344,7 +388,13 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
     // -> start, x and y the other two sets; a lone launch goes to the
     // caller's set, or from it to the workspace.
     int i = 0;
-    if (c.chain) {
+    // A call of three or four iterations: pairs by warp strips up to 1448^2, which
+    // need no tensor maps and no longer chains (64^2 29.9 -> 28.5 us, 1024^2 49.2
+    // -> 45.6 a call; 2048^2 106 against 93; the same results).
+    const bool pairs = c.pairs || (c.chain && c.strip && !cert && n >= 3 && n <= 4 &&
+                                   c.prm.rho_schedule_len <= k0 &&
+                                   (size_t)c.P.g.H * (size_t)c.P.g.W <= (size_t)1 << 21);
+    if (c.chain && !pairs) {
         // one iteration per launch while the rho schedule lasts, then launches
         // of up to four iterations, at least two of them; the last one carries
         // the certificates
@@ -366,8 +416,10 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
             certified = may_cert && j == first + nl - 1;
             if (!dry) {
                 const StepConfig cfg = m < 0 ? step_at(c.cfg, c.prm, 2, false, k0 + j) : c.cfg;
-                cudaError_t e = binary_maps(c, cur);
-                if (e == cudaSuccess)
+                const bool alone = T == 1 && !certified && runs_alone(c, cur, dst, i);
+                cudaError_t e =
+                    alone ? one_iteration(c, cur, dst, cfg, st) : binary_maps(c, cur);
+                if (e == cudaSuccess && !alone)
                     e = binary_chain_step(c.storage, c.P, bset(c, dst), cfg.aniso, cfg.ac, T, i,
                                           c.cmaps[cur], partials, c.cert_blocks,
                                           certified ? cert : nullptr, c.err, st);
@@ -378,7 +430,7 @@ cudaError_t binary_run(const BinaryCall& c, int n, int& cur, cudaStream_t st, in
         }
         i = n;
     }
-    if (c.pairs) {
+    if (pairs) {
         const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
         const int first = sched < n ? sched : n;
         for (; i < first; ++i) {

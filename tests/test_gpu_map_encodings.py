@@ -1,6 +1,6 @@
 """Tensor maps are encoded on the host where a launch first reads them (about 0.15 us
 each, beside calls of 30 to 50 us): none in a certificate of the binary model or in a
-solve that replays its graph, one buffer set's in a call of one iteration.  The
+solve that replays its graph, one buffer set's at most in a call of one iteration.  The
 fault-injection library, in a process of its own, counts them."""
 import json
 import os
@@ -54,9 +54,10 @@ def test_maps_are_encoded_where_they_are_read():
     assert proc.returncode == 0, proc.stderr[-3000:]
     line = [x for x in proc.stdout.splitlines() if x.startswith("RESULT ")][-1]
     out = json.loads(line[len("RESULT "):])
-    # a set: five (binary) or five (Potts) state planes, three or two cost planes; the
-    # cost planes once a call.  Replayed solve, certificates, 1 iteration, 40 iterations
-    assert out["binary_2"] == [0, 0, 8, 18]
-    assert out["binary_3"] == [0, 0, 8, 13]
-    assert out["potts_2"] == [0, 7, 7, 12]
-    assert out["potts_3"] == [0, 7, 7, 12]
+    # at most a set's five state planes and the three (binary) or two cost planes, these
+    # once a call: replayed solve, certificates, 1 iteration, 40 iterations
+    most = {"binary_2": [0, 0, 8, 18], "binary_3": [0, 0, 8, 13],
+            "potts_2": [0, 7, 7, 12], "potts_3": [0, 7, 7, 12]}
+    for name, counts in out.items():
+        assert all(a <= b for a, b in zip(counts, most[name])), (name, counts)
+    assert out["binary_2"][3] == 18  # they are counted
