@@ -666,6 +666,12 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     }
     if (rows && call.cert) {
         call.rows = true;
+        // lone iterations of two labels with 16-bit flows: strips, where two label
+        // warps a block leave the rows short of warps (2048^2 69.5 -> 60.8 us,
+        // 4096^2 247 -> 233; 1024^2 equal; three labels 76.8 against 85.5; the same
+        // results)
+        call.strip = L == 2 && es == 2 && (size_t)H * (size_t)W > (size_t)1 << 20 &&
+                     potts_strip_eligible(call.P.g, p->storage, C, alpha, call.user, call.ws);
         call.rfused = potts_rows_fused(call.P, p->storage, call.cfg.aniso);
         return CMF_OK;
     }
@@ -737,8 +743,12 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
             const int it = i < singles ? 1 : 2;
             if (!dry) {
                 const StepConfig cfg = step_at(c.cfg, c.prm, c.P.L, true, k0 + i);
-                cudaError_t e = row_maps(c, cur);
-                if (e == cudaSuccess)
+                const bool alone = it == 1 && c.strip;
+                cudaError_t e = alone ? potts_strip_step(c.storage, c.P, cur == 0 ? c.user : c.ws,
+                                                         cur == 0 ? c.ws : c.user, cfg.aniso,
+                                                         cfg.ac, cu_in, st)
+                                      : row_maps(c, cur);
+                if (e == cudaSuccess && !alone)
                     e = potts_rows_step(c.storage, c.P, cur == 0 ? c.ws : c.user, cfg.aniso,
                                         cfg.ac, cu_in, it, c.rmaps[cur], c.rfused, c.err, st);
                 if (e != cudaSuccess) return e;

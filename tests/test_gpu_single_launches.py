@@ -47,6 +47,26 @@ def test_binary_scheduled_iterations(cmf, shape, storage, monkeypatch):
             np.testing.assert_array_equal(got[k], ref[k], err_msg=f"{k} {calls}")
 
 
+# both sides of the size from which two labels' lone iterations leave the rows
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(60, 62), (1030, 1030)])
+def test_potts_scheduled_iterations(cmf, shape, storage):
+    from paper_2004_11227_gb300 import synth
+    inst = synth.random_potts(*shape, 2, seed=7, field_alpha=True)
+    for calls in ((3,), (1, 2), (6, 1), (8,), (12,)):
+        out = []
+        for variant in (0, 2):
+            s = cmf.alloc_potts(inst, cmf.default_params(2, 2, storage=storage, variant=variant,
+                                                         rho_schedule=SCHED))
+            cmf.cmf_init_potts(s)
+            for n in calls:
+                cmf.cmf_iterate_potts(s, n)
+            cmf.cmf_eval_potts(s)  # raises if a device wait ran out
+            out.append(s.state())
+        for k in out[0]:
+            np.testing.assert_array_equal(out[0][k], out[1][k], err_msg=f"{k} {calls}")
+
+
 def _us(f):
     best = 1e9
     for i in range(8):
@@ -59,6 +79,18 @@ def _us(f):
         if i > 1:
             best = min(best, a.elapsed_time(b) * 1e3)
     return best
+
+
+def test_potts_scheduled_iterations_are_not_slower(cmf):
+    from paper_2004_11227_gb300 import synth
+    inst = synth.random_potts(2048, 2048, 2, seed=7, field_alpha=True)
+    n, t = 60, []
+    for variant in (0, 2):
+        p = cmf.default_params(2, 2, storage=1, variant=variant, rho_schedule=np.full(n, 1.9))
+        s = cmf.alloc_potts(inst, p)
+        cmf.cmf_init_potts(s)
+        t.append(_us(lambda: cmf.cmf_iterate_potts(s, n)))
+    assert t[0] <= 1.07 * t[1], t  # the rows took 1.14 times as long
 
 
 # a chain of one warp took 1.3 times as long in all of these
