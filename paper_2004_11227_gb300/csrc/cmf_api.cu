@@ -659,12 +659,21 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
     const bool rows =
         free_choice && !call.cfg.dr &&
         potts_rows_eligible(call.P, p->storage, call.cfg.ac, call.user, call.ws);
-    call.cert = potts_rows_layout(call.P, p->storage, call.user, call.ws) && tma_available();
-    if (dr_rows && call.cert) {
+    const bool side =
+        potts_rows_layout(call.P, p->storage, call.user, call.ws) && tma_available();
+    // Certificates with the labels side by side, but for two labels in float32 at
+    // even widths between 1024^2 and 1448^2, where the strips' take 2 us less (an
+    // iteration and its check 69.7 -> 67.7 us and 115.7 -> 113.8; at 900^2 equal, at
+    // 724^2 and 2048^2 the strips' take 9 and 7 us more, with 16-bit flows, rPDRQ or
+    // more labels always more).
+    const size_t px = (size_t)H * (size_t)W;
+    call.cert = side && !(L == 2 && es == 4 && W % 2 == 0 && !call.cfg.dr &&
+                          px >= (size_t)1 << 20 && px <= (size_t)1 << 21);
+    if (dr_rows && side) {
         call.dr_rows = true;
         return CMF_OK;
     }
-    if (rows && call.cert) {
+    if (rows && side) {
         call.rows = true;
         // lone iterations of two labels with 16-bit flows: strips, where two label
         // warps a block leave the rows short of warps (2048^2 69.5 -> 60.8 us,
@@ -712,8 +721,8 @@ cudaError_t row_maps(const PottsCall& c, int i) {
 
 // The certificate launch for buffer set `set` (0 or 1): labels side by side
 // where the layout allows it (a call, host part included: 2048^2, L = 16
-// 547 -> 423 us, L = 4 197 -> 153 us; 721 x 1283, L = 8 199 -> 97 us; not
-// slower anywhere from 128^2 on), else the strip or tile kernel.
+// 619 -> 434 us, L = 4 195 -> 158 us; 721 x 1283, L = 8 199 -> 97 us; within a
+// solve 1 to 10 us less per check from 8^2 to 512^2), else the strip or tile kernel.
 cudaError_t potts_certify(const PottsCall& c, int set, cudaStream_t st, const EvalTail& T) {
     double* partials = (double*)(c.wsbase + c.w.partials);
     if (c.cert) {
