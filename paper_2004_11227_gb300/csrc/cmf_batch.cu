@@ -94,24 +94,8 @@ constexpr int kSideCols = 56;  // columns a strip of the labels side by side adv
 constexpr int kBaseRows = 12, kChainRows = 16, kMostBands = 8192;
 struct MergeRule {
     int rows[4];  // base band heights; 0: one band a block (params.batch_rows)
+    int used;     // instances it is for
 };
-// Base bands of `base` rows a block should take when the active instances have
-// `rows` strip rows in all: rounds of the blocks a GB300 holds, each costing the
-// band and the rows that fill and drain it; ties to shorter bands.
-__device__ int merge_for(long long rows, int base, int resident, int fill) {
-    const int f[9] = {1, 2, 3, 4, 6, 8, 12, 16, 22};
-    int best = 1;
-    long long cost = -1;
-    for (int k = 0; k < 9; ++k) {
-        const int r = base * f[k];
-        const long long c = ((rows + r - 1) / r + resident - 1) / resident * (r + fill);
-        if (cost < 0 || c < cost) {
-            cost = c;
-            best = f[k];
-        }
-    }
-    return best;
-}
 
 int potts_rows_for(int maxL) { return maxL <= 8 ? 4 : (maxL <= 16 ? 2 : 1); }
 
@@ -185,6 +169,8 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
     off += al(sizeof(int) * (size_t)(b.n_bin_tiles + b.n_potts_tiles + b.n_bin_ev + b.n_potts_ev + 4));
     b.items = off;
     off += al(sizeof(int2) * (size_t)(b.n_strip_items + b.n_chain_items + b.n_rows_items + 1));
+    b.maps = off;  // (what the host uploads ends here)
+    off += al(sizeof(BatchMaps) * (size_t)b.n_maps);
     b.partials = off;
     off += al(sizeof(double) * 3 * (size_t)(b.n_bin_ev + b.n_potts_ev + 1));
     b.scal = off;
@@ -193,8 +179,6 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
     off += al(64);
     b.states = off;
     for (int i = 0; i < n; ++i) off += state_bytes(inst[i], p.storage);
-    b.maps = off;
-    off += al(sizeof(BatchMaps) * (size_t)b.n_maps);
     b.total = off;
     return b;
 }
@@ -206,7 +190,15 @@ struct BatchCtl {
     int merge[4];  // base bands a block takes (three classes of label counts, chains)
 };
 
-// One block: how many base bands a block takes, from the instances still active.
+// Candidates for the base bands a block takes: 1, 2, 3, 4, 6, 8, 12, 16, 22.
+__device__ int merge_candidate(int f) {
+    return f < 8 ? (int)(0x100C080604030201ull >> 8 * f) & 255 : 22;
+}
+
+// One block: how many base bands a block takes, from the strip rows of the instances
+// still active: rounds of the blocks a GB300 holds, each costing the band and the rows
+// that fill and drain it; ties to shorter bands.  Sixteen threads a class, a
+// candidate each (one thread a class, a candidate after the other: 3 us a check).
 __device__ void set_merge(const BatchDesc* desc, int n, const MergeRule& rule, BatchCtl* ctl) {
     __shared__ unsigned long long rows[4];
     if (threadIdx.x < 4) rows[threadIdx.x] = 0;
@@ -219,13 +211,20 @@ __device__ void set_merge(const BatchDesc* desc, int n, const MergeRule& rule, B
         atomicAdd(&rows[k], (unsigned long long)D.sp_nstrips * (unsigned long long)H);
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
-        const int k = threadIdx.x;
-        ctl->merge[k] = rule.rows[k] == 0
-                            ? 1
-                            : merge_for((long long)rows[k], rule.rows[k],
-                                        k == 3 ? 152 * 4 : 152 * (3 - k), k == 3 ? 14 : 8);
+    if (threadIdx.x >= 64) return;
+    const int k = threadIdx.x >> 4, f = threadIdx.x & 15;
+    const int resident = k == 3 ? 152 * 4 : 152 * (3 - k), fill = k == 3 ? 14 : 8;
+    unsigned long long key = ~0ull;  // cost, then the candidate
+    if (f < 9 && rule.rows[k] > 0) {
+        const unsigned r = rule.rows[k] * merge_candidate(f);
+        const unsigned long long blocks = (rows[k] + r - 1) / r;
+        key = (blocks + resident - 1) / resident * (r + fill) * 16 + f;
     }
+    for (int d = 8; d > 0; d >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, d);
+        key = other < key ? other : key;
+    }
+    if (f == 0) ctl->merge[k] = rule.rows[k] > 0 ? merge_candidate(key & 15) : 1;
 }
 
 __global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl, MergeRule rule) {
@@ -237,9 +236,10 @@ __global__ void k_batch_reset(BatchDesc* desc, int n, BatchCtl* ctl, MergeRule r
     if (threadIdx.x == 0) {
         ctl->it = 0;
         ctl->stop = 0;
+        ctl->err = 0;
     }
     __syncthreads();
-    set_merge(desc, n, rule, ctl);
+    if (rule.used) set_merge(desc, n, rule, ctl);
 }
 
 // One block per instance: sum its certificate partials in index order.
@@ -284,7 +284,7 @@ __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, Batch
                                cudaGraphConditionalHandle h, int set_h) {
     const int it = ctl->it + K;
     const bool failed = ctl->err == kErrWaitTimeout;
-    int any = 0;
+    int any = 0, left = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         BatchDesc& D = desc[i];
         if (!D.active) continue;
@@ -307,9 +307,11 @@ __global__ void k_batch_decide(BatchDesc* desc, int n, const double* scal, Batch
         } else {
             any = 1;
         }
+        if (!D.active) left = 1;
     }
     any = __syncthreads_or(any);
-    set_merge(desc, n, rule, ctl);
+    left = __syncthreads_or(left);
+    if (rule.used && any && left) set_merge(desc, n, rule, ctl);
     if (threadIdx.x == 0) {
         ctl->it = it;
         ctl->stop = any ? 0 : 1;
@@ -506,11 +508,6 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     double* partials = (double*)(ws + B.partials);
     double* scal = (double*)(ws + B.scal);
     BatchCtl* ctl = (BatchCtl*)(ws + B.ctl);
-    CMF_CUDA_TRY(cudaMemcpyAsync(d_desc, desc.data(), sizeof(BatchDesc) * n,
-                                 cudaMemcpyHostToDevice, st));
-    if (!all.empty())
-        CMF_CUDA_TRY(cudaMemcpyAsync(tables, all.data(), sizeof(int) * all.size(),
-                                     cudaMemcpyHostToDevice, st));
     // one table after the other: the Potts items first (their finalize launch
     // takes them all), then the chains'
     std::vector<int2> table;
@@ -523,14 +520,26 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     d_ritems[1] = d_ritems[0] + ritems[0].size();
     d_ritems[2] = d_ritems[1] + ritems[1].size();
     int2* d_citems = d_ritems[2] + ritems[2].size();
-    if (!table.empty())
-        CMF_CUDA_TRY(cudaMemcpyAsync(d_items, table.data(), sizeof(int2) * table.size(),
-                                     cudaMemcpyHostToDevice, st));
     BatchMaps* d_maps = (BatchMaps*)(ws + B.maps);
-    if (!maps.empty())
-        CMF_CUDA_TRY(cudaMemcpyAsync(d_maps, maps.data(), sizeof(BatchMaps) * maps.size(),
-                                     cudaMemcpyHostToDevice, st));
-    CMF_CUDA_TRY(cudaMemsetAsync(&ctl->err, 0, sizeof(int), st));
+    // descriptors, tables and tensor maps are neighbours in the workspace: in one
+    // copy where they are small (a copy costs about 5 us, the smallest batches 80 to
+    // 130 in all), else one each (gathering 65 KB first cost more than it saved)
+    const size_t up_bytes = (maps.empty() ? B.items + sizeof(int2) * table.size()
+                                          : B.maps + sizeof(BatchMaps) * maps.size()) - B.desc;
+    std::vector<char> up(up_bytes <= 32768 ? up_bytes : 0);
+    cudaError_t sent = cudaSuccess;
+    auto put = [&](size_t at, const void* src, size_t bytes) {
+        if (!bytes || sent != cudaSuccess) return;
+        if (!up.empty()) memcpy(up.data() + (at - B.desc), src, bytes);
+        else sent = cudaMemcpyAsync(ws + at, src, bytes, cudaMemcpyHostToDevice, st);
+    };
+    put(B.desc, desc.data(), sizeof(BatchDesc) * n);
+    put(B.tiles, all.data(), sizeof(int) * all.size());
+    put(B.items, table.data(), sizeof(int2) * table.size());
+    put(B.maps, maps.data(), sizeof(BatchMaps) * maps.size());
+    if (!up.empty())
+        sent = cudaMemcpyAsync(ws + B.desc, up.data(), up.size(), cudaMemcpyHostToDevice, st);
+    CMF_CUDA_TRY(sent);
     // cold starts
     if (!p->warm_start) {
         for (int i = 0; i < n; ++i) {
@@ -544,6 +553,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     MergeRule rule;
     for (int k = 0; k < 3; ++k) rule.rows[k] = B.rows_fixed ? 0 : B.rows_rows;
     rule.rows[3] = B.chain_rows;
+    rule.used = (int)maps.size();
     k_batch_reset<<<1, 256, 0, st>>>(d_desc, n, ctl, rule);
     CMF_CUDA_TRY(cudaGetLastError());
 
@@ -646,14 +656,13 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
         }
         return e;
     };
-    // the results, on the call's own stream
+    // the results, on the call's own stream (a device wait that ran out: the
+    // instances that were still iterating say so)
     auto collect = [&]() -> cmf_status {
-        int herr = 0;
-        CMF_CUDA_TRY(cudaMemcpyAsync(&herr, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, st));
         CMF_CUDA_TRY(cudaMemcpyAsync(desc.data(), d_desc, sizeof(BatchDesc) * n,
                                      cudaMemcpyDeviceToHost, st));
         CMF_CUDA_TRY(cudaStreamSynchronize(st));
-        bool all_ok = true;
+        bool all_ok = true, failed = false;
         for (int i = 0; i < n; ++i) {
             inst[i].iters = desc[i].iters;
             inst[i].status = desc[i].status;
@@ -662,8 +671,9 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             inst[i].gap = desc[i].gap;
             inst[i].res = desc[i].res;
             all_ok = all_ok && desc[i].status == CMF_OK;
+            failed = failed || desc[i].status == CMF_ETIMEOUT;
         }
-        if (herr == kErrWaitTimeout) return CMF_ETIMEOUT;
+        if (failed) return CMF_ETIMEOUT;
         return all_ok ? CMF_OK : CMF_NOT_CONVERGED;
     };
     if (!p->use_graph) {
@@ -687,7 +697,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
     do {
         if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) break;
         bool made = true;
-        for (size_t t = 0; t < tracks.size() && made; ++t) {
+        for (size_t t = 0; tracks.size() > 1 && t < tracks.size() && made; ++t) {
             cudaEvent_t x = nullptr;
             made = cudaEventCreateWithFlags(&x, cudaEventDisableTiming) == cudaSuccess;
             if (made) ev.push_back(x);
