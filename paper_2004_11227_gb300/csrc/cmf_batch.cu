@@ -34,7 +34,7 @@ struct BatchLayout {
     int n_bin_tiles, n_potts_tiles, n_bin_ev, n_potts_ev, potts_rows, max_l, n_strip_items;
     // instances on the single solves' kernels (chains of warps; labels side by
     // side, classes of at most 4, 8 and 16 labels)
-    bool chains;
+    bool chains, binary_chains;
     int n_maps, n_chain_items, chain_rows;
     int n_rows_items;  // room for their items (at bands of at most 12 rows)
     int rows_rows, rows_labels[3];
@@ -69,8 +69,19 @@ Grid grid_of(const cmf_instance& in) {
     return Grid{in.H, in.W, in.pitch, (size_t)in.H * (size_t)in.pitch};
 }
 int rows_class(int L) { return L <= 4 ? 0 : (L <= 8 ? 1 : 2); }
+// Labels side by side, but for large grids of two labels whose chunks hold many
+// launches of one iteration (both of two, two of six where check_every / 2 is odd):
+// those stay on warp strips (2 x 1024^2, 60 iterations by strips / side by side, ms:
+// checks every 2 float32 7.2 / 8.2, float16 6.4 / 7.9, every 10 float16 3.6 / 4.0,
+// float32 4.15 / 3.97; at 256^2 side by side is 1.7 to 2.7 times as fast).
 bool batch_side(const cmf_instance& in, const cmf_params& p) {
     if (in.model != 1 || !relaxed_admm(p)) return false;
+    const size_t px = (size_t)in.H * (size_t)in.W;
+    if (in.L == 2 && in.W % 2 == 0 && px >= (size_t)1 << 20 && batch_strip(in, p) &&
+        (p.check_every == 2 ||
+         (p.storage != CMF_F32 && p.check_every <= 10 && p.check_every / 2 % 2 &&
+          px <= (size_t)1 << 21)))
+        return false;
     const PottsProblem P{in.d_cost, in.L, Alpha{in.d_alpha, in.alpha0}, grid_of(in), nullptr,
                          nullptr};
     const PottsStateV s{in.d_u, in.d_qx, in.d_qy, in.d_p, (float*)in.d_ps};
@@ -82,6 +93,20 @@ bool batch_chain(const cmf_instance& in, const cmf_params& p) {
     const BinProblem P{in.d_cost, in.d_cost + G.plane, Alpha{in.d_alpha, in.alpha0}, G};
     const BinStateV s{in.d_u, in.d_qx, in.d_qy, in.d_ps, in.d_p};
     return binary_chain_eligible(P, p.storage, s, s, s);
+}
+// Whether the binary instances run by chains: a chunk is an even number of launches,
+// and short ones cost nearly as much as long ones (16 x 128^2, float32: one iteration
+// 17.6 us, four 24.8, on tiles one 12.8).  100 iterations, tiles / chains, ms: checks
+// every 2, 16 x 128^2 1.72 / 2.60 and 16 x 512^2 10.9 / 13.5; every 4, 1.30 / 1.56 and
+// 9.3 / 6.9; every 10, 1.05 / 1.16 (float16 1.08 / 1.03) and 8.2 / 5.2; every 20,
+// 1.01 / 0.95 and 8.0 / 4.2.  The states are the same.
+bool chains_pay(const cmf_instance* inst, int n, const cmf_params& p) {
+    const int K = p.check_every;
+    if (K >= 12 || (K >= 6 && p.storage != CMF_F32)) return true;
+    size_t px = 0;
+    for (int i = 0; i < n; ++i)
+        if (inst[i].model == 0) px += (size_t)inst[i].H * (size_t)inst[i].W;
+    return K >= 4 && px > (size_t)1 << 20;
 }
 constexpr int kSideCols = 56;  // columns a strip of the labels side by side advances
 // Base bands of the instances on the single solves' kernels: three classes of
@@ -112,6 +137,7 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
                          bool chains = true) {
     BatchLayout b{};
     b.chains = chains;
+    b.binary_chains = chains && chains_pay(inst, n, p);
     long long strip_rows_all = 0;
     for (int i = 0; chains && i < n; ++i) {
         const cmf_instance& in = inst[i];
@@ -141,7 +167,7 @@ BatchLayout batch_layout(const cmf_instance* inst, int n, const cmf_params& p,
         const int ntx = (in.W + 31) / 32;
         const int ev = ntx * ((in.H + 31) / 32);
         if (in.model == 0) {
-            if (chains && batch_chain(in, p)) {
+            if (b.binary_chains && batch_chain(in, p)) {
                 b.n_chain_items += (in.W + batch_chain_cols() - 1) / batch_chain_cols() *
                                    ((in.H + b.chain_rows - 1) / b.chain_rows);
                 ++b.n_maps;
@@ -367,8 +393,16 @@ extern "C" size_t cmf_batch_workspace_bytes(const cmf_instance* inst, int n, con
     if (!inst || n < 1 || !p || check_batch_params(p) != CMF_OK) return 0;
     for (int i = 0; i < n; ++i)
         if (check_instance(inst[i], *p) != CMF_OK) return 0;
-    const size_t a = batch_layout(inst, n, *p).total, b = batch_layout(inst, n, *p, false).total;
-    return a > b ? a : b;
+    // the same for every check interval (which kernels run depends on it): a batch
+    // may be solved with another one, and the autotuner tries several
+    size_t most = batch_layout(inst, n, *p, false).total;
+    for (int k : {2, 4, 10, 20}) {
+        cmf_params q = *p;
+        q.check_every = k;
+        const size_t t = batch_layout(inst, n, q).total;
+        most = t > most ? t : most;
+    }
+    return most;
 }
 
 extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_params* p,
@@ -438,7 +472,7 @@ extern "C" cmf_status cmf_solve_batch(cmf_instance* inst, int n, const cmf_param
             D.bw.pt = b;
             D.tile_base = (int)tb.size();
             D.ev_tab = (int)eb.size();
-            if (B.chains && batch_chain(in, *p)) {
+            if (B.binary_chains && batch_chain(in, *p)) {
                 D.sp_out = batch_chain_cols();
                 D.sp_nstrips = (in.W + D.sp_out - 1) / D.sp_out;
                 D.sp_rows = B.chain_rows;
