@@ -377,8 +377,9 @@ cmf_status cmf_solve_potts(const float *d_C, int L, const float *d_alpha, float 
 /* ------------------------------------------------------------------------ */
 /* Autotuning (no counterpart in the paper: a launch-configuration search).  */
 /* Solves the problem from a cold start once per candidate configuration --  */
-/* the kernel variant (0 (Potts), 1, 2, 4 (binary), 8, 16, 32) of the fused ADMM */
-/* algorithms, or the sRBGS sweep count (1, 2, 3) of fused rPDRQ, and with   */
+/* the kernel variant (1, 2, 8, 16, 32, and 4 for binary problems of even    */
+/* width or 0 for the others) of the fused ADMM algorithms, or the sRBGS     */
+/* sweep count (1, 2, 3) of fused rPDRQ, and with                            */
 /* p->tune_step = 1 the ADMM step size c (c, 2c, 4c, 8c) -- with everything  */
 /* else taken from *p, and writes the candidate with the shortest time to   */
 /* p->tol_gap                                                               */

@@ -1532,15 +1532,16 @@ cmf_status cmf_solve_potts(const float* d_C, int L, const float* d_alpha, float 
 namespace {
 
 // Candidate list for a parameter set: kernel variants of the fused ADMM path
-// and sRBGS sweep counts of the fused rPDRQ path.
-std::vector<cmf_params> tune_candidates(const cmf_params& p, bool binary) {
+// and sRBGS sweep counts of the fused rPDRQ path.  Binary problems run the chains
+// of warps under variant 4 at even widths, under variant 0 alone at odd ones.
+std::vector<cmf_params> tune_candidates(const cmf_params& p, bool binary, int W) {
     std::vector<cmf_params> out;
     const bool fused = p.impl == CMF_FUSED;
     const bool dr = p.algo == CMF_RPDRQ;
     std::vector<int> variants = {p.variant};
     std::vector<int> sweeps = {p.sweeps};
-    if (fused && !dr) variants = binary ? std::vector<int>{1, 2, 4, 8, 16, 32}
-                                        : std::vector<int>{0, 1, 2, 8, 16, 32};
+    if (fused && !dr) variants = binary && W % 2 == 0 ? std::vector<int>{1, 2, 4, 8, 16, 32}
+                                                      : std::vector<int>{0, 1, 2, 8, 16, 32};
     if (fused && dr) sweeps = {1, 2, 3};
     for (int v : variants)
         for (int s : sweeps) {
@@ -1575,7 +1576,7 @@ std::vector<cmf_params> tune_candidates(const cmf_params& p, bool binary) {
 }
 
 template <typename Solve>
-cmf_status tune_loop(const cmf_params* p, bool binary, Solve solve, cmf_params* best,
+cmf_status tune_loop(const cmf_params* p, bool binary, int W, Solve solve, cmf_params* best,
                      double* h_best_ms, cudaStream_t st) {
     if (!p || !best) return CMF_EINVAL;
     cudaEvent_t e0, e1;
@@ -1584,7 +1585,7 @@ cmf_status tune_loop(const cmf_params* p, bool binary, Solve solve, cmf_params* 
     double best_ms = 1e300;
     bool found = false;
     cmf_status last = CMF_EINVAL;
-    for (const cmf_params& q : tune_candidates(*p, binary)) {
+    for (const cmf_params& q : tune_candidates(*p, binary, W)) {
         cmf_status s = solve(q);  // warm-up (and validity check)
         last = s;
         if (s != CMF_OK) continue;
@@ -1620,7 +1621,7 @@ extern "C" cmf_status cmf_autotune_binary(const float* d_Cs, const float* d_Ct,
                                           void* d_ws, size_t ws_bytes, cmf_params* best,
                                           double* h_best_ms, void* stream) {
     return tune_loop(
-        p, true,
+        p, true, W,
         [&](const cmf_params& q) {
             return cmf_solve_binary(d_Cs, d_Ct, d_alpha, alpha0, H, W, pitch, &q, d_u, d_qx,
                                     d_qy, d_ps, d_pt, nullptr, 0, nullptr, d_ws, ws_bytes,
@@ -1636,7 +1637,7 @@ extern "C" cmf_status cmf_autotune_potts(const float* d_C, int L, const float* d
                                          size_t ws_bytes, cmf_params* best, double* h_best_ms,
                                          void* stream) {
     return tune_loop(
-        p, false,
+        p, false, W,
         [&](const cmf_params& q) {
             return cmf_solve_potts(d_C, L, d_alpha, alpha0, H, W, pitch, &q, d_u, d_qx, d_qy,
                                    d_p, d_ps, nullptr, 0, nullptr, d_ws, ws_bytes, stream);
