@@ -488,10 +488,15 @@ def cmf_autotune_potts(s: Potts, stream=None):
     return best, ms.value
 
 
+# Part of the tuning cache's keys, raised when the kernels behind the variants or the
+# candidates change: a choice made among others is searched for again.
+TUNE_GENERATION = 2
+
+
 def tuned_params(problem, cache_path: str | None = None) -> Params:
     """Autotuned parameters for a Binary / Potts container, cached in a JSON
     file keyed by (model, H, W, L, storage, algo, impl, tune_step, c,
-    phase_storage, phase_gap, SM count, device)."""
+    phase_storage, phase_gap, SM count, device, TUNE_GENERATION)."""
     import json
 
     p = problem.params
@@ -499,7 +504,8 @@ def tuned_params(problem, cache_path: str | None = None) -> Params:
     key = "|".join(str(v) for v in (
         "binary" if isinstance(problem, Binary) else "potts", problem.H, problem.W,
         getattr(problem, "L", 2), p.storage, p.algo, p.impl, p.tune_step, p.c,
-        p.phase_storage, p.phase_gap, props.multi_processor_count, props.name))
+        p.phase_storage, p.phase_gap, props.multi_processor_count, props.name,
+        f"kernels {TUNE_GENERATION}"))
     path = cache_path or os.environ.get(
         "CMF_TUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "cmf_tune.json"))
     try:
