@@ -323,9 +323,11 @@ __device__ __forceinline__ void potts_rows_block(const PottsRowsMaps& M, const P
         if (!ok && sums && lane == 0) {
             // a label never arrived (one that gives up does not): report it and
             // let the copies in flight land before the block's shared memory
-            // goes; the rows issued by then follow from the step
+            // goes; with two service warps the rows issued by then follow from
+            // the step
             atomicExch(err, kErrWaitTimeout);
-            const int n = min(k > 0 ? issued_after(k - 1) : kState, il + 1);
+            const int n =
+                min(!two ? issued : (k > 0 ? issued_after(k - 1) : kState), il + 1);
             for (int i = max(0, n - kAux); i < n; ++i)
                 mbar_wait(b_full + 8 * (i & (kAux - 1)), (i / kAux) & 1);
         }
