@@ -5,8 +5,8 @@
 // Instances whose layout allows it run the kernels of the single solves (chains
 // of warps; labels side by side, in classes of at most 4, 8 and 16 labels), each
 // kind on a branch of the graph of its own, since no kind waits for another.  The
-// rest (rPDRQ, more than 16 labels, layouts those kernels refuse, a workspace
-// without room for the tensor maps) run one kernel over the tiles of the binary
+// rest (rPDRQ, more than 16 labels, layouts those kernels refuse, check intervals
+// too short for them, a workspace without room for the tensor maps) run one kernel over the tiles of the binary
 // instances, one over the tiles of the Potts instances and one over their
 // warp-strip items; a block or warp maps its work to an instance through a
 // device table and skips it when that instance has converged.  Every

@@ -5,6 +5,14 @@
 // maps from device memory, and leaves at once when the instance has converged.
 // The tables hold one class of label counts each, so that small instances do
 // not pay for the largest block.
+//
+// What bounds it.  The problem's and the state's pointers come from memory and not
+// from the parameter bank: with two iterations a launch 118 registers for at most 4
+// labels (three blocks of 5 warps an SM instead of four), and 104 to 148 bytes a
+// thread spilled for 8 and 16 labels, where the single solves' kernel spills 4.  16
+// instances of 512^2, L = 4, float32: 286 us per launch (ncu, cold L2), 36% of the
+// issue slots, DRAM at 28%; the latency of loads and of a row's chain of shuffles is
+// the rest.
 #pragma once
 
 #include "cmf_binary_chain.cuh"

@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(32 * (kWarps + 1), 3)
             float qx_e, qy_e, ps_e, pt_e, qx_o, qy_o, ps_o, pt_o;
             binary_dr_flows<S, ANISO>(D, un.x, gx_e, gy_e, fx.x, fy.x, fs.x, ft.x, al.x, cs.x,
                                       ct.x, qx_e, qy_e, ps_e, pt_e);
-            // the strips' compiled code squares the odd columns' y first (float32)
+            // the strips' results add the odd columns' squares the other way round
+            // (float32)
             binary_dr_flows<S, ANISO, ES == 4>(D, un.y, gx_o, gy_o, fx.y, fy.y, fs.y, ft.y, al.y,
                                                cs.y, ct.y, qx_o, qy_o, ps_o, pt_o);
             PF::st(s1.u + o, un.x, un.y);

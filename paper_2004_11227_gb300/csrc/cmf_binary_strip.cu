@@ -1,6 +1,7 @@
 // Binary ADMM iteration by warp strips (Eq. rpADMMII, Eq. rpADMMI, pADMM-TY
-// Eq. ADMM:Tai_yuan): variant 2, and the single iterations of calls that run
-// cmf_binary_strip2.cu.  The rPDRQ strips below run variant 2, two to four
+// Eq. ADMM:Tai_yuan): variant 2, the single iterations of calls that run
+// cmf_binary_strip2.cu, and iterations that run alone beside the chains of warps
+// where a chain of one is slower (the rule is in cmf_api.cu).  The rPDRQ strips below run variant 2, two to four
 // sweeps, and rows or planes that are not 16-byte aligned (otherwise
 // cmf_binary_dr_rows.cu).
 //

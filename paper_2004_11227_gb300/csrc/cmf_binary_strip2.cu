@@ -1,8 +1,9 @@
 // Binary ADMM, two iterations per launch by warp strips (Eq. rpADMMII, Eq.
 // rpADMMI, pADMM-TY Eq. ADMM:Tai_yuan, ALG1 Eq. iteration:pd:seg): temporal
 // blocking of the one-iteration warp-strip kernel of cmf_binary_strip.cu.
-// Runs where the chains of warps (cmf_binary_chain.cuh) cannot: even widths whose
-// rows or planes are not 16-byte aligned.
+// Runs where the chains of warps (cmf_binary_chain.cuh) cannot, even widths whose
+// rows or planes are not 16-byte aligned, and calls of three or four iterations up
+// to 1448^2.
 #include "cmf_kernels.cuh"
 #include "cmf_strip.cuh"
 

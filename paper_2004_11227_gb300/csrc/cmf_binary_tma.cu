@@ -1,5 +1,6 @@
 // Binary ADMM iteration (Eq. rpADMMI / Eq. rpADMMII) as a persistent kernel
-// with TMA-staged tiles.
+// with TMA-staged tiles: variants 8, 16 and 32, and (16 rows) iterations that run
+// alone beside the chains of warps at odd widths up to 1024^2.
 //
 // Each block walks output tiles t = blockIdx.x, blockIdx.x + gridDim.x, ...
 // The five state planes it reads with a halo (q_x, q_y, p_s, p_t, u) arrive

@@ -23,10 +23,10 @@
 // thread instructions per label-pixel at 60% of the issue slots (583 us at
 // 2048^2, L = 16, float16; odd widths: tiles).  Here each plane is read once
 // (1.40 GB of DRAM reads for 1.38 GB) and the thresholds come from shared
-// memory: 118 thread instructions per label-pixel (two correctly rounded
+// memory: 137 thread instructions per label-pixel (two correctly rounded
 // square roots, two projections and two double-float sums per pair are most of
-// them), 54-58% of the issue slots, DRAM at 41-46%.  Measured (ncu): 2048^2,
-// L = 16 float32 381 us, L = 4 190 -> 117 us.
+// them), 61% of the issue slots, DRAM at 45%.  Measured at 2048^2, float32: L = 16
+// 390 us (ncu), a call 619 -> 434 us; L = 4 a call 195 -> 158 us.
 #pragma once
 
 #include "cmf_potts_rows.cuh"

@@ -1,7 +1,8 @@
 // Potts ADMM iteration by warp strips (Eq. multi:fg:4, the Eckstein-Bertsekas
 // Potts equations after Thm 2, and pADMM-TY, Eq. mADMM:Tai_yuan): variant 2,
-// more than 16 labels, costs made from the image, and rows or planes that are
-// not 16-byte aligned (otherwise cmf_potts_rows.cuh).
+// more than 16 labels, costs made from the image, rows or planes that are not
+// 16-byte aligned, and lone iterations of two labels with 16-bit flows above
+// 1024^2 (otherwise cmf_potts_rows.cuh).
 //
 // Work unit: one warp, a strip of 64 columns (two adjacent columns per lane)
 // and a band of R output rows.  The warp walks the labels one after another;
