@@ -607,7 +607,11 @@ struct PottsCall {
     bool rows;                   // fused ADMM, labels side by side, up to two iterations a launch
     bool cert;                   // certificates with the labels side by side
     bool dr_rows;                // rPDRQ with the labels side by side
-    PottsTmaMaps maps[2];        // tensor maps of the user / workspace state sets
+    // tensor maps of the user / workspace state sets (tma); with rows encoded where
+    // a launch first reads a set
+    mutable PottsTmaMaps maps[2];
+    mutable int tma_mapped = 0;  // the sets encoded, a bit each
+    int tma_rows;                // rows of a tile
     // tensor maps of the two sets (rows, dr_rows, cert), encoded by row_maps
     // where a launch first reads a set
     mutable PottsRowsMaps rmaps[2];
@@ -679,8 +683,16 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
         // warps a block leave the rows short of warps (2048^2 69.5 -> 60.8 us,
         // 4096^2 247 -> 233; 1024^2 equal; three labels 76.8 against 85.5; the same
         // results)
-        call.strip = L == 2 && es == 2 && (size_t)H * (size_t)W > (size_t)1 << 20 &&
+        call.strip = L == 2 && es == 2 && px > (size_t)1 << 20 &&
                      potts_strip_eligible(call.P.g, p->storage, C, alpha, call.user, call.ws);
+        // at odd widths, where a call is lone iterations throughout, TMA tiles up to
+        // 2^20 pixels (1024 x 1023 27.3 -> 25.0 us; 2048 x 2047 89 against 101)
+        if (L == 2 && es == 2 && W % 2 && px <= (size_t)1 << 20) {
+            call.tma_rows = potts_tma_auto_ty(p->storage, p->aniso, L);
+            call.tma = potts_tma_fits(p->storage, L, call.tma_rows) &&
+                       potts_tma_eligible(call.P.g, p->storage, call.user) &&
+                       potts_tma_eligible(call.P.g, p->storage, call.ws);
+        }
         call.rfused = potts_rows_fused(call.P, p->storage, call.cfg.aniso);
         return CMF_OK;
     }
@@ -703,6 +715,7 @@ cmf_status potts_prepare(const float* C, int L, const float* alpha, float alpha0
                        cudaSuccess &&
                    potts_tma_maps(call.P.g, L, p->storage, call.ws, ty, call.maps[1]) ==
                        cudaSuccess;
+        call.tma_mapped = 3;
     }
     if (!call.tma && !call.cfg.dr && !call.cfg.plain && p->variant >= 8)
         return CMF_EINVAL;  // TMA tiles requested but the layout does not allow them
@@ -741,12 +754,13 @@ cudaError_t potts_certify(const PottsCall& c, int set, cudaStream_t st, const Ev
 // one launch more (less than copying a state set back).
 cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int k0 = 0,
                       const EvalTail* cert = nullptr, bool dry = false, bool home = false) {
-    if (c.rows && n > 0) {
-        // single launches for the scheduled iterations and an odd remainder
-        const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
-        int singles = sched < n ? sched : n;
-        singles += (n - singles) % 2;
-        if (home && singles + 2 <= n && (singles + (n - singles) / 2) % 2) singles += 2;
+    // with two iterations a launch: single ones for the scheduled iterations and an
+    // odd remainder
+    const int sched = c.prm.rho_schedule_len > k0 ? c.prm.rho_schedule_len - k0 : 0;
+    int singles = sched < n ? sched : n;
+    singles += (n - singles) % 2;
+    if (home && singles + 2 <= n && (singles + (n - singles) / 2) % 2) singles += 2;
+    if (c.rows && n > 0 && !(c.tma && singles == n)) {
         float cu_in = 0.0f;  // the first launch reads u itself, later ones the w form
         for (int i = 0; i < n;) {
             const int it = i < singles ? 1 : 2;
@@ -817,8 +831,14 @@ cudaError_t potts_run(const PottsCall& c, int n, int& cur, cudaStream_t st, int 
                 return e;
         } else if (c.tma) {
             const PottsStateV& b = cur == 0 ? c.ws : c.user;
-            cudaError_t e = potts_admm_tma_step(c.storage, c.P, b, cfg.aniso, cfg.ac,
-                                                c.maps[cur], c.err, st);
+            cudaError_t e = cudaSuccess;
+            if (!(c.tma_mapped >> cur & 1)) {
+                e = potts_tma_maps(c.P.g, c.P.L, c.storage, cur == 0 ? c.user : c.ws, c.tma_rows,
+                                   c.maps[cur]);
+                if (e != cudaSuccess) return e;
+                c.tma_mapped |= 1 << cur;
+            }
+            e = potts_admm_tma_step(c.storage, c.P, b, cfg.aniso, cfg.ac, c.maps[cur], c.err, st);
             if (e != cudaSuccess) return e;
             cur ^= 1;
         } else {

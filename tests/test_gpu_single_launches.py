@@ -49,15 +49,18 @@ def test_binary_scheduled_iterations(cmf, shape, storage, monkeypatch):
 
 # both sides of the size from which two labels' lone iterations leave the rows
 @pytest.mark.parametrize("storage", [0, 1, 2])
-@pytest.mark.parametrize("shape", [(60, 62), (1030, 1030)])
+@pytest.mark.parametrize("shape", [(60, 62), (1030, 1030), (41, 61), (1000, 1001), (1030, 1031)])
 def test_potts_scheduled_iterations(cmf, shape, storage):
+    """Odd widths: against the TMA tiles of the automatic height, which the automatic
+    choice runs where the costs are float16 planes (here the same values)."""
     from paper_2004_11227_gb300 import synth
     inst = synth.random_potts(*shape, 2, seed=7, field_alpha=True)
+    inst.costs = inst.costs.astype(np.float16).astype(inst.costs.dtype)
     for calls in ((3,), (1, 2), (6, 1), (8,), (12,)):
         out = []
-        for variant in (0, 2):
-            s = cmf.alloc_potts(inst, cmf.default_params(2, 2, storage=storage, variant=variant,
-                                                         rho_schedule=SCHED))
+        for kw in (dict(), dict(costs=2) if shape[1] % 2 else dict(variant=2)):
+            s = cmf.alloc_potts(inst, cmf.default_params(2, 2, storage=storage,
+                                                         rho_schedule=SCHED, **kw))
             cmf.cmf_init_potts(s)
             for n in calls:
                 cmf.cmf_iterate_potts(s, n)
@@ -81,16 +84,18 @@ def _us(f):
     return best
 
 
-def test_potts_scheduled_iterations_are_not_slower(cmf):
+# the rows took 1.14 and 1.09 times as long
+@pytest.mark.parametrize("shape,other", [((2048, 2048), 2), ((1024, 1023), 16)])
+def test_potts_scheduled_iterations_are_not_slower(cmf, shape, other):
     from paper_2004_11227_gb300 import synth
-    inst = synth.random_potts(2048, 2048, 2, seed=7, field_alpha=True)
+    inst = synth.random_potts(*shape, 2, seed=7, field_alpha=True)
     n, t = 60, []
-    for variant in (0, 2):
+    for variant in (0, other):
         p = cmf.default_params(2, 2, storage=1, variant=variant, rho_schedule=np.full(n, 1.9))
         s = cmf.alloc_potts(inst, p)
         cmf.cmf_init_potts(s)
         t.append(_us(lambda: cmf.cmf_iterate_potts(s, n)))
-    assert t[0] <= 1.07 * t[1], t  # the rows took 1.14 times as long
+    assert t[0] <= 1.06 * t[1], t
 
 
 # a chain of one warp took 1.3 times as long in all of these
